@@ -78,7 +78,9 @@ typedef struct {
                                  default 10065.32 */
     int newton_terms;         /* Stumpff series terms in the Newton phase: 8 (default,
                                  Sec. 3.2) or 6 (Appendix A).  The Halley phase always
-                                 uses 4 terms; 2 Halley + 2 Newton iterations (Sec. 3.2).
+                                 uses 4 terms; 2 Halley + 2 Newton iterations (Sec. 3.2),
+                                 the Newton phase as one third-order step in fixed point
+                                 wherever that reaches the same solution.
                                  T terms: c_2, c_3 summed through the z^T term,
                                  c_n(z) ~ sum_{k=0..T} (-z)^k / (n+2k)!.  The initial
                                  guess is X = h/r0. */
@@ -103,16 +105,12 @@ typedef struct {
                                  instead of J(dt/2) I(dt) J(dt/2): J and I commute when there
                                  is no GR term (Sec. 3.1), so this is the same map up to
                                  rounding, one jump cheaper.  Ignored when gr_mode != 0. */
-    int halley_fp32;          /* 1: the Kepler solver's initial guess and its 2 Halley steps
-                                 (Sec. 3.2) run in FP32; the 2 Newton steps, the f and g
-                                 functions and everything else stay FP64.  The Halley phase
-                                 only supplies the Newton phase's start, and two FP64 Newton
-                                 steps from a start within ~1e-7 converge quadratically to
-                                 FP64 rounding, so inside the solver's domain (Fig. 1) the
-                                 results match the all-FP64 solver to rounding.  Outside it
-                                 (pericentre timescale below ~2 steps) both are inaccurate and
-                                 may stop differently.  Default 0: the whole solver in FP64
-                                 (the paper's arithmetic). */
+    int halley_fp32;          /* 0 (default) or 1; has no effect on results or speed.  The Kepler
+                                 solver starts from two Halley steps (Sec. 3.2) in FP32 either
+                                 way: they only supply the starting point, after which one step
+                                 in 64-bit fixed point reaches the solution to ~2^-58
+                                 (csrc/whg_fixed.cuh).  Outside that solver's domain the
+                                 fixed-iteration solver runs in FP64 throughout. */
     int repack_frozen;        /* -1 (default): on when a stop rule is on
                                  (close_encounter_hill > 0 or eject_factor > 0), else off.
                                  1: every graph_launches step launches (every 16 without

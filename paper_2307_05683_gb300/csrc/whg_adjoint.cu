@@ -379,8 +379,10 @@ __device__ __forceinline__ void loss_body(const WhgState& st, const WhgBuckets& 
     const double dt = pl.has_sys ? st.dt[s] : 1.0e-3;
     const long long ns = pl.has_sys ? st.nstep[s] : 0;
     const bool real = pl.has_sys && g.p < st.nplan[s];
-    double sx = qx, sy = qy, sz = qz, svx = vx, svy = vy, svz = vz, X = 0.0;
-    if (ns > 0) kepler_drift<NT>(mu, 0.5 * dt, sx, sy, sz, svx, svy, svz, X, st.halley32 != 0);
+    double sx = qx, sy = qy, sz = qz, svx = vx, svy = vy, svz = vz;
+    DriftVals dv{};
+    if (ns > 0) kepler_drift<NT, true>(mu, 0.5 * dt, sx, sy, sz, svx, svy, svz, &dv);
+    const double X = dv.X;
     const int u = pl.has_sys ? user_index(st, s) : 0;
     double ex = 0.0, ey = 0.0, ez = 0.0;
     if (real) {
@@ -441,9 +443,9 @@ __device__ __forceinline__ void tape_body(const WhgState& st, const WhgBuckets& 
         tp[kTQ0 * NL] = qx; tp[(kTQ0 + 1) * NL] = qy; tp[(kTQ0 + 2) * NL] = qz;
         tp[kTV0 * NL] = vx; tp[(kTV0 + 1) * NL] = vy; tp[(kTV0 + 2) * NL] = vz;
         const double h = (s0 + k == 0) ? 0.5 * dt : dt;
-        double X;
         DriftVals dv;
-        kepler_drift<NT, true>(mu, h, qx, qy, qz, vx, vy, vz, X, st.halley32 != 0, &dv);
+        kepler_drift<NT, true>(mu, h, qx, qy, qz, vx, vy, vz, &dv);
+        const double X = dv.X;
         {
             const KeplerCoef kc = kepler_vjp_coef<NT>(mu, X, dv);
             const double* kv = reinterpret_cast<const double*>(&kc);

@@ -409,7 +409,6 @@ int whg_create(whg_ctx** out, int n_systems, int max_planets, const whg_options*
     st.hill = opt.close_encounter_hill;
     st.eject = opt.eject_factor;
     st.merge = (opt.merge_jumps && opt.gr_mode == 0) ? 1 : 0;
-    st.halley32 = opt.halley_fp32 ? 1 : 0;
     st.full_rotation = opt.interaction_schedule == 1 ? 1 : 0;
 
     if (opt.queue_steps > 0) {                           // counter, per-group flags, error flag

@@ -27,6 +27,7 @@
 
 #include <stdint.h>
 
+#include "whg_fixed.cuh"
 #include "whg_internal.h"
 
 #define WHG_FULL_MASK 0xffffffffu
@@ -250,40 +251,6 @@ __device__ __forceinline__ double rsqrt_pow(double x)
 __device__ __forceinline__ double rsqrt(double x) { return rsqrt_pow<false>(x); }
 __device__ __forceinline__ double rsqrt_cubed(double x) { return rsqrt_pow<true>(x); }
 
-// FP64 -> FP32 from the bit fields (sign, exponent rebiased from 1023 to
-// 127, mantissa truncated to 23 bits) on the integer pipe: the hardware
-// conversion runs on the FP64 pipe, the scarce unit here.  Rounds toward
-// zero; |x| below the FP32 normal range gives a signed zero, above it (and
-// inf, NaN) a signed infinity.
-__device__ __forceinline__ float to_f32(double x)
-{
-    const unsigned hi = (unsigned)__double2hiint(x);
-    const unsigned lo = (unsigned)__double2loint(x);
-    const unsigned sign = hi & 0x80000000u;
-    const int ex = (int)((hi >> 20) & 0x7ffu) - 1023 + 127;            // FP32 biased exponent
-    unsigned b = sign | ((unsigned)ex << 23) | ((hi & 0x000fffffu) << 3) | (lo >> 29);
-    b = ex <= 0 ? sign : b;
-    b = ex >= 255 ? (sign | 0x7f800000u) : b;
-    return __uint_as_float(b);
-}
-
-// FP32 -> FP64 from the bit fields (exact for normal numbers; subnormals give
-// a signed zero; inf and NaN stay inf and NaN), on the integer pipe.
-__device__ __forceinline__ double to_f64(float f)
-{
-    const unsigned b = __float_as_uint(f);
-    const unsigned sign = b & 0x80000000u;
-    const unsigned ex = (b >> 23) & 0xffu;
-    const unsigned man = b & 0x007fffffu;
-    unsigned hi = sign | ((ex + 896u) << 20) | (man >> 3);
-    unsigned lo = man << 29;
-    hi = ex == 0u ? sign : hi;
-    lo = ex == 0u ? 0u : lo;
-    hi = ex == 255u ? (sign | 0x7ff00000u | (man ? 0x00080000u : 0u)) : hi;
-    lo = ex == 255u ? 0u : lo;
-    return __hiloint2double((int)hi, (int)lo);
-}
-
 __device__ __forceinline__ bool is_finite(double x)
 {
     return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000;
@@ -327,34 +294,11 @@ __device__ __forceinline__ void stumpff_c2c3(double z, double& c2, double& c3)
     StumpffHorner<T - 1>::run(z, c2, c3);
 }
 
-// The same series in FP32 (coefficients 1/k! rounded to float), for the
-// Halley phase's starting point only.
-template <int K>
-struct StumpffHornerF {
-    static __device__ __forceinline__ void run(float z, float& c2, float& c3)
-    {
-        c2 = fmaf(-z, c2, (float)(1.0 / Factorial<2 * K + 2>::value));
-        c3 = fmaf(-z, c3, (float)(1.0 / Factorial<2 * K + 3>::value));
-        StumpffHornerF<K - 1>::run(z, c2, c3);
-    }
-};
-template <>
-struct StumpffHornerF<-1> {
-    static __device__ __forceinline__ void run(float, float&, float&) {}
-};
-
-template <int T>
-__device__ __forceinline__ void stumpff_c2c3_f32(float z, float& c2, float& c3)
-{
-    c2 = (float)(1.0 / Factorial<2 * T + 2>::value);
-    c3 = (float)(1.0 / Factorial<2 * T + 3>::value);
-    StumpffHornerF<T - 1>::run(z, c2, c3);
-}
-
-
 // ------------------------------------------------------------------------
 // Kepler drift of one planet for time h under H_K,i (Sec. 3.2, Eq. 3),
-// mu = G m0.  Universal variable X solves Kepler's equation
+// mu = G m0: kepler_general, the fixed-iteration solver in FP64, for the
+// drifts outside the fixed-point solver's domain.  Universal variable X solves
+// Kepler's equation
 //     F(X)  = r0 G1 + eta0 G2 + mu G3 - h = r0 X + eta0 G2 + zeta0 G3 - h = 0,
 //     F'(X) = r = r0 + eta0 G1 + zeta0 G2,
 //     F''   = eta0 G0 + zeta0 G1
@@ -365,26 +309,20 @@ __device__ __forceinline__ void stumpff_c2c3_f32(float z, float& c2, float& c3)
 // the final X = X1 + d come from the values at the last Newton point X1 by
 // one Taylor step (dG_n/dX = G_{n-1}); |d| is the last Newton correction, so
 // the neglected d^2 terms are far below rounding.  Then the Lagrange f - 1,
-// g, fdot, gdot - 1.
-// h32 (uniform across the warp) runs the initial guess and the Halley phase
-// in FP32: they only supply the Newton phase's starting point, and from a
-// start within ~1e-7 two FP64 Newton steps reach FP64 rounding
-// (quadratic convergence: 1e-7 -> 1e-14 -> rounding), so the result keeps
-// FP64 accuracy wherever the FP64 Halley phase converges, while ~60 FP64
-// operations per drift move to the FP32 pipe.  No other branches.
-// Returns beta > 0; Xout receives the final universal variable.  With
-// VALS, *dv also receives the drift's intermediate values (for the adjoint's
-// tape); the arithmetic is the same either way.
+// g, fdot, gdot - 1.  No branches.
+// Returns beta > 0.  With VALS, *dv also receives the drift's intermediate
+// values (for the adjoint's tape); the arithmetic is the same either way.
 struct DriftVals {
+    double X;                            // universal variable of the solution
     double r0i, r0, eta0, beta;          // of the initial state
     double G1, G2, G3;                   // Stiefel functions at the final X
     double ri, A, fm1, g, fd, gdm1;      // 1/r, mu/r0, Lagrange coefficients
 };
 
-template <int NT, bool VALS = false>
-__device__ __forceinline__ bool kepler_drift(double mu, double h, double& qx, double& qy,
+template <int NT, bool VALS>
+__device__ __forceinline__ bool kepler_general(double mu, double h, double& qx, double& qy,
                                              double& qz, double& vx, double& vy, double& vz,
-                                             double& Xout, bool h32 = false, DriftVals* dv = nullptr)
+                                             DriftVals* dv)
 {
     const double r0sq = fma(qx, qx, fma(qy, qy, qz * qz));
     const double r0i = rsqrt(r0sq);
@@ -394,40 +332,20 @@ __device__ __forceinline__ bool kepler_drift(double mu, double h, double& qx, do
     const double beta = fma(2.0 * mu, r0i, -v2);
     const double zeta0 = fma(-beta, r0, mu);
     double X, X2, c2, c3, G1, G2, G3;
-    if (h32) {
-        const float r0f = to_f32(r0), r0if = to_f32(r0i), eta0f = to_f32(eta0);
-        const float zeta0f = to_f32(zeta0), betaf = to_f32(beta), hf = to_f32(h);
-        const float beta_eta0f = betaf * eta0f, beta_zeta0f = betaf * zeta0f;
-        float Xs = hf * r0if;
+    X = h * r0i;
 #pragma unroll
-        for (int it = 0; it < 2; ++it) {             // Halley (FP32)
-            const float Y2 = Xs * Xs;
-            float s2, s3;
-            stumpff_c2c3_f32<4>(betaf * Y2, s2, s3);
-            const float H2 = Y2 * s2, H3 = (Y2 * Xs) * s3;
-            const float F = fmaf(r0f, Xs, fmaf(eta0f, H2, fmaf(zeta0f, H3, -hf)));
-            const float Fp = fmaf(zeta0f, H2, fmaf(-beta_eta0f, H3, fmaf(eta0f, Xs, r0f)));
-            const float Fpp = fmaf(-beta_zeta0f, H3, fmaf(-beta_eta0f, H2, fmaf(zeta0f, Xs, eta0f)));
-            const float den = fmaf(-0.5f * F, Fpp, Fp * Fp);
-            Xs = Xs - __fdividef(F * Fp, den);
-        }
-        X = to_f64(Xs);
-    } else {
-        X = h * r0i;
-#pragma unroll
-        for (int it = 0; it < 2; ++it) {             // Halley
-            X2 = X * X;
-            stumpff_c2c3<4>(beta * X2, c2, c3);
-            G2 = X2 * c2;
-            G3 = (X2 * X) * c3;
-            G1 = fma(-beta, G3, X);
-            const double G0 = fma(-beta, G2, 1.0);
-            const double F = fma(r0, X, fma(eta0, G2, fma(zeta0, G3, -h)));
-            const double Fp = fma(zeta0, G2, fma(eta0, G1, r0));
-            const double Fpp = fma(zeta0, G1, eta0 * G0);
-            const double den = fma(neg_half(F), Fpp, Fp * Fp);   // (2F'^2 - F F'') / 2
-            X = fma(-(F * Fp), rcp(den), X);
-        }
+    for (int it = 0; it < 2; ++it) {             // Halley
+        X2 = X * X;
+        stumpff_c2c3<4>(beta * X2, c2, c3);
+        G2 = X2 * c2;
+        G3 = (X2 * X) * c3;
+        G1 = fma(-beta, G3, X);
+        const double G0 = fma(-beta, G2, 1.0);
+        const double F = fma(r0, X, fma(eta0, G2, fma(zeta0, G3, -h)));
+        const double Fp = fma(zeta0, G2, fma(eta0, G1, r0));
+        const double Fpp = fma(zeta0, G1, eta0 * G0);
+        const double den = fma(neg_half(F), Fpp, Fp * Fp);   // (2F'^2 - F F'') / 2
+        X = fma(-(F * Fp), rcp(den), X);
     }
     double d = 0.0;
 #pragma unroll
@@ -462,8 +380,8 @@ __device__ __forceinline__ bool kepler_drift(double mu, double h, double& qx, do
     vy = fma(fd, qy, fma(gdm1, vy, vy));
     vz = fma(fd, qz, fma(gdm1, vz, vz));
     qx = nqx; qy = nqy; qz = nqz;
-    Xout = Xf;
     if constexpr (VALS) {
+        dv->X = Xf;
         dv->r0i = r0i; dv->r0 = r0; dv->eta0 = eta0; dv->beta = beta;
         dv->G1 = G1f; dv->G2 = G2f; dv->G3 = G3f;
         dv->ri = ri; dv->A = mr0; dv->fm1 = fm1; dv->g = g; dv->fd = fd; dv->gdm1 = gdm1;
@@ -471,13 +389,79 @@ __device__ __forceinline__ bool kepler_drift(double mu, double h, double& qx, do
     return beta > 0.0;
 }
 
-template <int NT>
-__device__ __forceinline__ bool kepler_drift(double mu, double h, double& qx, double& qy,
-                                             double& qz, double& vx, double& vy, double& vz,
-                                             bool h32 = false)
+// kepler_general as one out-of-line function for all callers: it is rarely
+// run, and inlined it would hold registers and code of every step kernel.
+template <bool VALS>
+struct GeneralDrift {
+    double qx, qy, qz, vx, vy, vz;
+    DriftVals dv;
+    bool bound;
+};
+template <>
+struct GeneralDrift<false> {
+    double qx, qy, qz, vx, vy, vz;
+    bool bound;
+};
+
+template <int NT, bool VALS>
+__device__ __noinline__ GeneralDrift<VALS> kepler_general_call(double mu, double h, double qx, double qy, double qz,
+                                                               double vx, double vy, double vz)
 {
-    double X;
-    return kepler_drift<NT>(mu, h, qx, qy, qz, vx, vy, vz, X, h32);
+    GeneralDrift<VALS> r;
+    DriftVals dv;
+    r.bound = kepler_general<NT, VALS>(mu, h, qx, qy, qz, vx, vy, vz, &dv);
+    r.qx = qx; r.qy = qy; r.qz = qz;
+    r.vx = vx; r.vy = vy; r.vz = vz;
+    if constexpr (VALS) r.dv = dv;
+    return r;
+}
+
+// The drift: the solution of Kepler's equation in fixed point (whg_fixed.cuh)
+// inside that solver's domain, which holds every resolved bound orbit, else
+// kepler_general.  The choice depends on the planet's own state only, so
+// results do not depend on which lane or warp holds it.  21 FP64
+// instructions (three scalar products and the new vectors) against 153.
+template <int NT, bool VALS = false>
+__device__ __forceinline__ bool kepler_drift(double mu, double h, double& qx, double& qy, double& qz, double& vx,
+                                             double& vy, double& vz, DriftVals* dv = nullptr)
+{
+    const double r0sq = fma(qx, qx, fma(qy, qy, qz * qz));
+    const double eta0 = fma(qx, vx, fma(qy, vy, qz * vz));
+    const double v2 = fma(vx, vx, fma(vy, vy, vz * vz));
+    fixed::Solution o;
+    if (!fixed::solve<NT, VALS>(mu, h, r0sq, eta0, v2, o)) {
+        const GeneralDrift<VALS> r = kepler_general_call<NT, VALS>(mu, h, qx, qy, qz, vx, vy, vz);
+        qx = r.qx; qy = r.qy; qz = r.qz;
+        vx = r.vx; vy = r.vy; vz = r.vz;
+        if constexpr (VALS) *dv = r.dv;
+        return r.bound;
+    }
+    if constexpr (VALS) {
+        const double r0i = rsqrt(r0sq);
+        const double w = h * r0i, w2 = w * w;
+        dv->X = o.s * w;
+        dv->r0i = r0i;
+        dv->r0 = r0sq * r0i;
+        dv->eta0 = eta0;
+        dv->beta = fma(2.0 * mu, r0i, -v2);
+        dv->G1 = o.g1 * w;
+        dv->G2 = o.g2 * w2;
+        dv->G3 = o.g3 * (w2 * w);
+        dv->ri = o.Ri * r0i;
+        dv->A = mu * r0i;
+        dv->fm1 = -o.fm1n;
+        dv->g = o.g;
+        dv->fd = -o.fdn;
+        dv->gdm1 = -o.gdm1n;
+    }
+    const double nqx = fma(-o.fm1n, qx, fma(o.g, vx, qx));
+    const double nqy = fma(-o.fm1n, qy, fma(o.g, vy, qy));
+    const double nqz = fma(-o.fm1n, qz, fma(o.g, vz, qz));
+    vx = fma(-o.fdn, qx, fma(-o.gdm1n, vx, vx));
+    vy = fma(-o.fdn, qy, fma(-o.gdm1n, vy, vy));
+    vz = fma(-o.fdn, qz, fma(-o.gdm1n, vz, vz));
+    qx = nqx; qy = nqy; qz = nqz;
+    return true;
 }
 
 // ------------------------------------------------------------------------
@@ -906,7 +890,6 @@ __device__ __forceinline__ void step_body(const WhgState& st, const WhgBuckets& 
     const double jc = (0.5 * dt) / mu;
     const double mrat = m / mu;
     const double kgr = GRM ? (-6.0 * mu * mu * dt) / (st.c_light * st.c_light) : 0.0;
-    const bool h32 = st.halley32 != 0;
     const bool full = st.full_rotation != 0;
     // close-encounter distances of this lane's pairs (once per launch)
     double thr2[4] = {0.0, 0.0, 0.0, 0.0};
@@ -931,7 +914,7 @@ __device__ __forceinline__ void step_body(const WhgState& st, const WhgBuckets& 
         const double hK = (nstep0 + done == 0) ? 0.5 * dt : dt;
         const double r0sq = fma(qx, qx, fma(qy, qy, qz * qz));
         const bool far = __double_as_longlong(r0sq) > __double_as_longlong(rej2);
-        const bool bound = kepler_drift<NT>(mu, hK, qx, qy, qz, vx, vy, vz, h32);
+        const bool bound = kepler_drift<NT>(mu, hK, qx, qy, qz, vx, vy, vz);
         bool close;
         if (GRM == 0 && st.merge) {                   // J(dt) I(dt): J and I commute without GR
             jump<L>(g, m, 2.0 * jc, vx, vy, vz, qx, qy, qz);
@@ -986,7 +969,7 @@ __device__ __forceinline__ void read_body(const WhgState& st, const WhgBuckets& 
     const double mu = pl.has_sys ? st.m0[s] : 1.0;
     const double dt = pl.has_sys ? st.dt[s] : 1.0e-3;
     const long long ns = pl.has_sys ? st.nstep[s] : 0;
-    if (ns > 0) kepler_drift<NT>(mu, 0.5 * dt, qx, qy, qz, vx, vy, vz, st.halley32 != 0);
+    if (ns > 0) kepler_drift<NT>(mu, 0.5 * dt, qx, qy, qz, vx, vy, vz);
     const double sqx = group_sum<L>(g, m * qx), sqy = group_sum<L>(g, m * qy), sqz = group_sum<L>(g, m * qz);
     const double spx = group_sum<L>(g, m * vx), spy = group_sum<L>(g, m * vy), spz = group_sum<L>(g, m * vz);
     if (!pl.has_sys) return;                         // after the last shuffle
@@ -1037,7 +1020,7 @@ __device__ __forceinline__ void energy_body(const WhgState& st, const WhgBuckets
     const double mu = pl.has_sys ? st.m0[s] : 1.0;
     const double dt = pl.has_sys ? st.dt[s] : 1.0e-3;
     if (pl.has_sys && st.nstep[s] > 0)
-        kepler_drift<NT>(mu, 0.5 * dt, qx, qy, qz, vx, vy, vz, st.halley32 != 0);
+        kepler_drift<NT>(mu, 0.5 * dt, qx, qy, qz, vx, vy, vz);
     const double r2 = fma(qx, qx, fma(qy, qy, qz * qz));
     double pair = 0.0;
 #pragma unroll

@@ -34,7 +34,6 @@ struct WhgState {
     double hill;                     // close-encounter rule: mutual Hill radii (0 = off)
     double eject;                    // ejection rule: factor on the largest initial a (0 = off)
     int merge;                       // one J(dt) before I(dt) (GR off only)
-    int halley32;                    // Kepler solver: initial guess and Halley phase in FP32
     int full_rotation;               // interaction: all L-1 rotations, no third-law reactions
     long long nl;                    // lane capacity of the lane arrays
     unsigned* dbg;                   // bounds-check flag word (debug builds only, else null)
