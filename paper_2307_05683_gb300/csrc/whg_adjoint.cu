@@ -248,6 +248,47 @@ __device__ __forceinline__ void prefetch_l2(const double* p)
     asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
 
+// The factors of the kick's vector-Jacobian product that do not depend on the
+// adjoints, from the positions during the kick: pair round r (partner j at
+// distance k = r + 1 <= L/2, this lane i) at p[(8r + n) NL], n = 0..7:
+// Q_j - Q_i (3), hm_j r^-3, hm_i r^-3, 3 hm_j r^-5, 3 hm_i r^-5, dt r^-3; the
+// GR factors at p[(32 + n) NL]: c = kgr/|Q|^4, 4 c/|Q|^2, 2 c/m0.
+constexpr int kKickTapeRound = 8;
+
+template <int L, int GRM>
+__device__ __forceinline__ void kick_tape(const Group<L>& g, double qx, double qy, double qz, double hm, double dt,
+                                          double kgr, double two_muinv, double* p, size_t NL)
+{
+#pragma unroll
+    for (int k = 1; 2 * k <= L; ++k) {
+        const int to = g.at(k);
+        const double dx = __shfl_sync(WHG_FULL_MASK, qx, to) - qx;   // Q_j - Q_i
+        const double dy = __shfl_sync(WHG_FULL_MASK, qy, to) - qy;
+        const double dz = __shfl_sync(WHG_FULL_MASK, qz, to) - qz;
+        const double hmj = __shfl_sync(WHG_FULL_MASK, hm, to);
+        const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
+        const double r3 = rsqrt_cubed(r2);
+        double* t = p + (size_t)(kKickTapeRound * (k - 1)) * NL;
+        const double r5x3 = 3.0 * (r3 * rcp(r2));
+        t[0] = dx;
+        t[NL] = dy;
+        t[2 * NL] = dz;
+        t[3 * NL] = hmj * r3;
+        t[4 * NL] = hm * r3;
+        t[5 * NL] = hmj * r5x3;
+        t[6 * NL] = hm * r5x3;
+        t[7 * NL] = dt * r3;
+    }
+    if (GRM != 0) {
+        const double r2 = fma(qx, qx, fma(qy, qy, qz * qz));
+        const double c = kgr * rcp_sq(r2);
+        double* t = p + (size_t)(4 * kKickTapeRound) * NL;
+        t[0] = c;
+        t[NL] = 4.0 * c * rcp(r2);
+        t[2 * NL] = c * two_muinv;
+    }
+}
+
 // Tape layout: per lane and step, WHG_TAPE_W doubles at stride NL.  Besides
 // the state the back kernel needs (velocities for the jumps, positions for
 // the GR term, the drift input), the tape holds everything of the kick and
@@ -256,14 +297,14 @@ __device__ __forceinline__ void prefetch_l2(const double* p)
 // dt r^-3, the GR factors, and the Kepler coefficients.
 constexpr int kTV3 = 0;        // v after the kick (input of the second jump)
 constexpr int kTQ2 = 3;        // Q during the kick
-constexpr int kTRound = 6;     // 4 rounds x 8 pair factors (see KickTape), written by kick()
-constexpr int kTGR = 38;       // c = kgr/|Q|^4, 4 c/|Q|^2, 2 c/m0, written by kick()
+constexpr int kTRound = 6;     // 4 rounds x 8 pair factors, written by kick_tape()
+constexpr int kTGR = 38;       // c = kgr/|Q|^4, 4 c/|Q|^2, 2 c/m0, written by kick_tape()
 constexpr int kTV1 = 41;       // v after the drift (input of the first jump)
 constexpr int kTQ0 = 44;       // drift input Q0
 constexpr int kTV0 = 47;       // drift input v0
 constexpr int kTKC = 50;       // KeplerCoef
 static_assert(kTKC + kKeplerCoefs == WHG_TAPE_W, "tape layout");
-static_assert(kTGR == kTRound + 4 * kKickTapeRound, "kick() writes its GR factors after 4 rounds");
+static_assert(kTGR == kTRound + 4 * kKickTapeRound, "kick_tape() writes its GR factors after 4 rounds");
 
 // Adjoint of the interaction kick (+GR) from the tape, with lambda_v the
 // adjoint of the velocities after it (which pass through unchanged).  Per
@@ -430,8 +471,7 @@ __device__ __forceinline__ void tape_body(const WhgState& st, const WhgBuckets& 
     const double mu = pl.has_sys ? st.m0[s] : 1.0;
     const double dt = pl.has_sys ? st.dt[s] : 1.0e-3;
     const bool real = pl.has_sys && g.p < st.nplan[s];
-    const double hm = dt * m, c = (0.5 * dt) / mu, mrat = m / mu;
-    const double kgr = GRM ? (-6.0 * mu * mu * dt) / (st.c_light * st.c_light) : 0.0;
+    const Masses<L> mc = masses_of<L, GRM>(g, real, m, mu, dt, st.c_light, GRM == 0 && st.merge, st.full_rotation != 0);
     const double* ck = adj.ckpt + (size_t)seg * 6 * NL;
     double qx = ck[0 * NL + lane], qy = ck[1 * NL + lane], qz = ck[2 * NL + lane];
     double vx = ck[3 * NL + lane], vy = ck[4 * NL + lane], vz = ck[5 * NL + lane];
@@ -453,13 +493,11 @@ __device__ __forceinline__ void tape_body(const WhgState& st, const WhgBuckets& 
             for (int i = 0; i < kKeplerCoefs; ++i) tp[(kTKC + i) * NL] = kv[i];
         }
         tp[kTV1 * NL] = vx; tp[(kTV1 + 1) * NL] = vy; tp[(kTV1 + 2) * NL] = vz;
-        const bool merged = GRM == 0 && st.merge;
-        jump<L>(g, m, merged ? 2.0 * c : c, vx, vy, vz, qx, qy, qz);
-        tp[kTQ2 * NL] = qx; tp[(kTQ2 + 1) * NL] = qy; tp[(kTQ2 + 2) * NL] = qz;
-        const KickTape kt{tp + (size_t)kTRound * NL, NL, dt, 2.0 / mu};
-        kick<L, GRM, true>(g, qx, qy, qz, hm, mrat, kgr, nothr, vx, vy, vz, st.full_rotation != 0, &kt);
+        double q2[3];
+        interact<L, GRM, true>(g, mc, pl.has_sys, qx, qy, qz, vx, vy, vz, nothr, false, q2);
+        tp[kTQ2 * NL] = q2[0]; tp[(kTQ2 + 1) * NL] = q2[1]; tp[(kTQ2 + 2) * NL] = q2[2];
+        kick_tape<L, GRM>(g, q2[0], q2[1], q2[2], mc.hm, dt, mc.kgr, 2.0 / mu, tp + (size_t)kTRound * NL, NL);
         tp[kTV3 * NL] = vx; tp[(kTV3 + 1) * NL] = vy; tp[(kTV3 + 2) * NL] = vz;
-        if (!merged) jump<L>(g, m, c, vx, vy, vz, qx, qy, qz);
         if (!real) {                                  // lanes without a planet stay parked
             qx = pqx; qy = pqy; qz = pqz;
             vx = pvx; vy = pvy; vz = pvz;

@@ -27,10 +27,16 @@
 
 #include <stdint.h>
 
-#include "whg_fixed.cuh"
+#include "whg_interact.cuh"
 #include "whg_internal.h"
 
 #define WHG_FULL_MASK 0xffffffffu
+
+// Blocks of WHG_MAX_BLOCK threads that the step kernels leave room for on an SM:
+// 2 (128 registers a thread, 16 resident warps) against 1 (160-186 registers,
+// 10-12 warps): 8192 8-planet systems 1.03e9 against 0.90e9 system-steps/s,
+// 65,536 1.15e9 against 1.09e9.
+#define WHG_STEP_BLOCKS 2
 
 namespace whg {
 
@@ -423,13 +429,14 @@ __device__ __noinline__ GeneralDrift<VALS> kepler_general_call(double mu, double
 // instructions (three scalar products and the new vectors) against 153.
 template <int NT, bool VALS = false>
 __device__ __forceinline__ bool kepler_drift(double mu, double h, double& qx, double& qy, double& qz, double& vx,
-                                             double& vy, double& vz, DriftVals* dv = nullptr)
+                                             double& vy, double& vz, DriftVals* dv = nullptr, bool live = true)
 {
     const double r0sq = fma(qx, qx, fma(qy, qy, qz * qz));
     const double eta0 = fma(qx, vx, fma(qy, vy, qz * vz));
     const double v2 = fma(vx, vx, fma(vy, vy, vz * vz));
     fixed::Solution o;
     if (!fixed::solve<NT, VALS>(mu, h, r0sq, eta0, v2, o)) {
+        if (!live) return false;
         const GeneralDrift<VALS> r = kepler_general_call<NT, VALS>(mu, h, qx, qy, qz, vx, vy, vz);
         qx = r.qx; qy = r.qy; qz = r.qz;
         vx = r.vx; vy = r.vy; vz = r.vz;
@@ -552,11 +559,23 @@ __device__ __forceinline__ void group_sum3(const Group<L>& g, double x, double y
 // products and 2 additions when every lane first forms its whole m x).
 // Each partial sum is formed by one lane only, and the last round adds a
 // pair's two values in both lanes (commutative), so every lane still ends
-// with the same bits.
+// with the same bits.  k: this lane's component before it is gathered (L = 4, 8).
+struct MassSum {
+    double k, x, y, z;
+};
+
 template <int L>
-__device__ __forceinline__ void group_msum3(const Group<L>& g, double m, double x, double y, double z,
-                                            double& sx, double& sy, double& sz)
+__device__ __forceinline__ void gather3(const Group<L>& g, double k, double& x, double& y, double& z)
 {
+    x = __shfl_sync(WHG_FULL_MASK, k, g.base);
+    y = __shfl_sync(WHG_FULL_MASK, k, g.base + L / 4);
+    z = __shfl_sync(WHG_FULL_MASK, k, g.base + L / 2);
+}
+
+template <int L>
+__device__ __forceinline__ MassSum mass_sum(const Group<L>& g, double m, double x, double y, double z)
+{
+    MassSum s;
     if (L == 4 || L == 8) {
         constexpr int H = L / 2, Q = L / 4;
         const bool hi = (g.p & H) != 0;          // keeps (z, 0), else (x, y)
@@ -571,12 +590,12 @@ __device__ __forceinline__ void group_msum3(const Group<L>& g, double m, double 
         double k = mid ? k1 : k0;
         k += __shfl_xor_sync(WHG_FULL_MASK, mid ? k0 : k1, Q);
         if (L == 8) k += __shfl_xor_sync(WHG_FULL_MASK, k, 1);
-        sx = __shfl_sync(WHG_FULL_MASK, k, g.base);
-        sy = __shfl_sync(WHG_FULL_MASK, k, g.base + Q);
-        sz = __shfl_sync(WHG_FULL_MASK, k, g.base + H);
+        s.k = k;
+        gather3<L>(g, k, s.x, s.y, s.z);
     } else {
-        group_sum3<L>(g, m * x, m * y, m * z, sx, sy, sz);
+        group_sum3<L>(g, m * x, m * y, m * z, s.x, s.y, s.z);
     }
+    return s;
 }
 
 // Jump step (Sec. 3.4, Eq. 6): Q_i += (h/m0) sum_j m_j v_j; jc = h / m0.
@@ -584,11 +603,10 @@ template <int L>
 __device__ __forceinline__ void jump(const Group<L>& g, double m, double jc, double vx, double vy,
                                      double vz, double& qx, double& qy, double& qz)
 {
-    double px, py, pz;
-    group_msum3<L>(g, m, vx, vy, vz, px, py, pz);
-    qx = fma(jc, px, qx);
-    qy = fma(jc, py, qy);
-    qz = fma(jc, pz, qz);
+    const MassSum P = mass_sum<L>(g, m, vx, vy, vz);
+    qx = fma(jc, P.x, qx);
+    qy = fma(jc, P.y, qy);
+    qz = fma(jc, P.z, qz);
 }
 
 // Interaction kick (Sec. 3.3, Eq. 5) plus the GR term, for time dt, added
@@ -607,41 +625,10 @@ __device__ __forceinline__ void jump(const Group<L>& g, double m, double jc, dou
 // evaluated by both of its lanes: 7 reciprocal square roots per lane for
 // L = 8); the close-encounter test then uses the distances k <= L/2, which
 // cover every pair from one side.
-// With GEOM (the adjoint's tape kernel), the factors of the kick's
-// vector-Jacobian product that do not depend on the adjoints are written to
-// kt: pair round r (partner j at distance k = r + 1 <= L/2, this lane i) at
-// kt.p[(8r + n) kt.NL], n = 0..7: Q_j - Q_i (3), hm_j r^-3, hm_i r^-3,
-// 3 hm_j r^-5, 3 hm_i r^-5, dt r^-3; the GR factors at kt.p[(32 + n) kt.NL]:
-// c = kgr/|Q|^4, 4 c/|Q|^2, 2 c/m0.  The velocities come out the same.
-struct KickTape {
-    double* p;
-    size_t NL;
-    double dt, two_muinv;
-};
-constexpr int kKickTapeRound = 8;
-
-template <bool GEOM>
-__device__ __forceinline__ void kick_geom(const KickTape* kt, int round, double dx, double dy, double dz,
-                                          double r2, double r3, double hmj, double hmi)
-{
-    if constexpr (GEOM) {
-        double* t = kt->p + (size_t)(kKickTapeRound * round) * kt->NL;
-        const double r5x3 = 3.0 * (r3 * rcp(r2));
-        t[0] = dx;
-        t[kt->NL] = dy;
-        t[2 * kt->NL] = dz;
-        t[3 * kt->NL] = hmj * r3;
-        t[4 * kt->NL] = hmi * r3;
-        t[5 * kt->NL] = hmj * r5x3;
-        t[6 * kt->NL] = hmi * r5x3;
-        t[7 * kt->NL] = kt->dt * r3;
-    }
-}
-
-template <int L, int GRM, bool GEOM = false>
+template <int L, int GRM>
 __device__ __forceinline__ bool kick(const Group<L>& g, double qx, double qy, double qz, double hm,
                                      double mrat, double kgr, const double* thr2, double& vx,
-                                     double& vy, double& vz, bool full = false, const KickTape* kt = nullptr)
+                                     double& vy, double& vz, bool full)
 {
     bool close = false;
     if (full) {
@@ -655,7 +642,6 @@ __device__ __forceinline__ bool kick(const Group<L>& g, double qx, double qy, do
             const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
             if (2 * k <= L) close |= __double_as_longlong(r2) < __double_as_longlong(thr2[k - 1]);
             const double r3 = rsqrt_cubed(r2);
-            if (2 * k <= L) kick_geom<GEOM>(kt, k - 1, dx, dy, dz, r2, r3, hmj, hm);
             const double sj = hmj * r3;
             vx = fma(sj, dx, vx);
             vy = fma(sj, dy, vy);
@@ -672,7 +658,6 @@ __device__ __forceinline__ bool kick(const Group<L>& g, double qx, double qy, do
             const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
             close |= __double_as_longlong(r2) < __double_as_longlong(thr2[k - 1]);
             const double r3 = rsqrt_cubed(r2);
-            kick_geom<GEOM>(kt, k - 1, dx, dy, dz, r2, r3, hmj, hm);
             const double sj = hmj * r3;
             vx = fma(sj, dx, vx);
             vy = fma(sj, dy, vy);
@@ -695,7 +680,6 @@ __device__ __forceinline__ bool kick(const Group<L>& g, double qx, double qy, do
             const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
             close |= __double_as_longlong(r2) < __double_as_longlong(thr2[L / 2 - 1]);
             const double r3 = rsqrt_cubed(r2);
-            kick_geom<GEOM>(kt, L / 2 - 1, dx, dy, dz, r2, r3, hmj, hm);
             const double sj = hmj * r3;
             vx = fma(sj, dx, vx);
             vy = fma(sj, dy, vy);
@@ -706,12 +690,6 @@ __device__ __forceinline__ bool kick(const Group<L>& g, double qx, double qy, do
         // a_GR(Q) = -6 (G m0)^2 Q / (c^2 |Q|^4); kgr = -6 m0^2 dt / c^2.
         const double r2 = fma(qx, qx, fma(qy, qy, qz * qz));
         const double c = kgr * rcp_sq(r2);
-        if constexpr (GEOM) {
-            double* t = kt->p + (size_t)(4 * kKickTapeRound) * kt->NL;
-            t[0] = c;
-            t[kt->NL] = 4.0 * c * rcp(r2);
-            t[2 * kt->NL] = c * kt->two_muinv;
-        }
         if (GRM == 1) {
             vx = fma(c, qx, vx);
             vy = fma(c, qy, vy);
@@ -725,6 +703,281 @@ __device__ __forceinline__ bool kick(const Group<L>& g, double qx, double qy, do
             vz = vz + (az - bz);
         }
     }
+    return close;
+}
+
+// ------------------------------------------------------------------------
+// J(dt/2) I(dt) J(dt/2) (merged: J(dt) I(dt)) of a system's planets.
+
+// What the sub-step needs that stays the same over a launch.
+template <int L>
+struct Masses {
+    double m, hm, mrat, jc, kgr;         // mass, dt m, m/m0, jump coefficient, GR coefficient
+    pairs::Pair hmp, kgp;                // hm and kgr as float pairs
+    pairs::Pair hmj[L > 1 ? L / 2 : 1];  // hm of the partners at distance 1..L/2
+    unsigned pairs_on;                   // bit k: the partner at distance k holds a planet, and so does this lane
+    bool real, full, merged;             // real: this lane holds a planet
+};
+
+template <int L, int GRM>
+__device__ __forceinline__ Masses<L> masses_of(const Group<L>& g, bool real, double m, double mu, double dt,
+                                               double c_light, bool merged, bool full)
+{
+    Masses<L> k;
+    k.m = m;
+    k.hm = dt * m;
+    k.mrat = m / mu;
+    k.jc = (0.5 * dt) / mu;
+    k.kgr = GRM ? (-6.0 * mu * mu * dt) / (c_light * c_light) : 0.0;
+    k.hmp = pairs::split(k.hm);
+    k.kgp = pairs::split(k.kgr);
+    k.real = real;
+    k.full = full;
+    k.merged = merged;
+    const unsigned reals = __ballot_sync(WHG_FULL_MASK, real);
+    k.pairs_on = 0u;
+#pragma unroll
+    for (int d = 1; 2 * d <= L; ++d) {
+        const int to = g.at(d);
+        k.hmj[d - 1].h = __shfl_sync(WHG_FULL_MASK, k.hmp.h, to);
+        k.hmj[d - 1].l = __shfl_sync(WHG_FULL_MASK, k.hmp.l, to);
+        k.pairs_on |= real ? ((reals >> to) & 1u) << d : 0u;
+    }
+    return k;
+}
+
+// The sub-step in FP64, for the systems that the float-pair form leaves out
+// (and the interaction schedule without reactions).  Out of line: rarely run.
+// Warp shuffles inside: every lane calls it.
+struct SubStep {
+    double m, hm, mrat, jc, kgr;
+    double qx, qy, qz, vx, vy, vz;           // in and out
+    double q2[3], thr2[4];                   // out: position during the kick; in: see kick()
+    bool full, merged, close;
+};
+
+template <int L, int GRM>
+__device__ __noinline__ void interact_general(SubStep* r)
+{
+    const Group<L> g;
+    double qx = r->qx, qy = r->qy, qz = r->qz, vx = r->vx, vy = r->vy, vz = r->vz;
+    // merged: J(dt) I(dt); J and I commute without GR
+    jump<L>(g, r->m, r->merged ? 2.0 * r->jc : r->jc, vx, vy, vz, qx, qy, qz);
+    r->q2[0] = qx; r->q2[1] = qy; r->q2[2] = qz;
+    r->close = kick<L, GRM>(g, qx, qy, qz, r->hm, r->mrat, r->kgr, r->thr2, vx, vy, vz, r->full);
+    if (!r->merged) jump<L>(g, r->m, r->jc, vx, vy, vz, qx, qy, qz);
+    r->qx = qx; r->qy = qy; r->qz = qz;
+    r->vx = vx; r->vy = vy; r->vz = vz;
+}
+
+// Float sums of (x, y, z) over the system's lanes: this lane's component
+// (L = 4, 8: returned in x) or all three in every lane.
+template <int L>
+__device__ __forceinline__ void sum_floats(const Group<L>& g, float& x, float& y, float& z)
+{
+    if (L == 4 || L == 8) {
+        constexpr int H = L / 2, Q = L / 4;
+        const bool hi = (g.p & H) != 0;
+        const float k0 = (hi ? z : x) + __shfl_xor_sync(WHG_FULL_MASK, hi ? x : z, H);
+        const float k1 = (hi ? 0.0f : y) + __shfl_xor_sync(WHG_FULL_MASK, hi ? y : 0.0f, H);
+        const bool mid = (g.p & Q) != 0;
+        float k = mid ? k1 : k0;
+        k += __shfl_xor_sync(WHG_FULL_MASK, mid ? k0 : k1, Q);
+        if (L == 8) k += __shfl_xor_sync(WHG_FULL_MASK, k, 1);
+        x = k;
+    } else if (L > 1) {
+        float sx = 0.0f, sy = 0.0f, sz = 0.0f;   // in lane order, the same bits in every lane
+#pragma unroll
+        for (int j = 0; j < L; ++j) {
+            const int from = g.in_group ? g.base + j : g.lane;
+            sx += __shfl_sync(WHG_FULL_MASK, x, from);
+            sy += __shfl_sync(WHG_FULL_MASK, y, from);
+            sz += __shfl_sync(WHG_FULL_MASK, z, from);
+        }
+        x = sx; y = sy; z = sz;
+    }
+}
+
+// The largest non-negative x of the system's lanes.
+template <int L>
+__device__ __forceinline__ int group_max(const Group<L>& g, int x)
+{
+    int r = x;
+    if ((L & (L - 1)) == 0) {
+#pragma unroll
+        for (int o = 1; o < L; o <<= 1) r = max(r, __shfl_xor_sync(WHG_FULL_MASK, r, o));
+    } else {
+#pragma unroll
+        for (int k = 1; k < L; ++k) r = max(r, __shfl_sync(WHG_FULL_MASK, x, g.at(k)));
+    }
+    return r;
+}
+
+// The sub-step with the kick's terms in float pairs (whg_interact.cuh).  Pair
+// rounds as in kick(): distances k < L/2 evaluated by the lower lane of the
+// rotation with the reaction passed back, distance L/2 by both lanes.  The
+// second jump uses that pair kicks leave sum m v unchanged (Newton's third
+// law): its sum is the first one's plus that of the GR kick, which is ~1e-8
+// of it and taken in floats (an error of 1e-15 of the jump's 1e-3 of the
+// position).  Returns false where the form does not hold (for a real lane);
+// the state is then unspecified.
+template <int L, int GRM, bool Q2>
+__device__ __forceinline__ bool interact_pairs(const Group<L>& g, const Masses<L>& c, double& qx, double& qy, double& qz,
+                                               double& vx, double& vy, double& vz, const double* thr2, bool hill,
+                                               bool& close, double* q2)
+{
+    const MassSum P = mass_sum<L>(g, c.m, vx, vy, vz);
+    const double jc = c.merged ? 2.0 * c.jc : c.jc;
+    qx = fma(jc, P.x, qx);
+    qy = fma(jc, P.y, qy);
+    qz = fma(jc, P.z, qz);
+    if (Q2) {
+        q2[0] = qx; q2[1] = qy; q2[2] = qz;
+    }
+    bool ok = true;
+    if (L > 1 || GRM != 0) {
+        // the common grid
+        const fixed::u64 bx = fixed::bits_of(qx), by = fixed::bits_of(qy), bz = fixed::bits_of(qz);
+        const int ex = fixed::exponent_of(bx), ey = fixed::exponent_of(by), ez = fixed::exponent_of(bz);
+        const int ev = max(fixed::exponent_of(fixed::bits_of(vx)),
+                           max(fixed::exponent_of(fixed::bits_of(vy)), fixed::exponent_of(fixed::bits_of(vz))));
+        const int eq = group_max<L>(g, c.real ? max(ex, max(ey, ez)) : 0);
+        const int K2 = 2 * (1040 - eq);                      // velocity changes are in 2^-K2
+        const int el = ev - 1023 - K2;
+        ok = (unsigned)(eq - 1007) <= 56u && (unsigned)(el + 60) <= 120u;
+        const float vl = fixed::bits_to_f32((unsigned)(127 + el) << 23);   // the velocity's scale
+        const pairs::Coord X = pairs::chunks(c.real ? fixed::to_fixed(bx, 5 + eq - ex) : (long long)(32 + g.p) << 54);
+        const pairs::Coord Y = pairs::chunks(fixed::to_fixed(by, 5 + eq - ey));
+        const pairs::Coord Z = pairs::chunks(fixed::to_fixed(bz, 5 + eq - ez));
+        pairs::Pair ax = {0.0f, 0.0f}, ay = {0.0f, 0.0f}, az = {0.0f, 0.0f};
+        // a term is accepted up to 2^-11 of the velocity, and weaker for
+        // separations where the grid shows (below 2^-7 of its extent)
+        auto accept = [](const pairs::Separation& s, float w, float v) {
+            return fmaxf(pairs::mul(w, pairs::mul(s.r2, s.y1)), pairs::mul(w, 128.0f)) <= pairs::mul(v, 1.0f / 2048.0f);
+        };
+#pragma unroll
+        for (int k = 1; 2 * k <= L; ++k) {
+            const int to = g.at(k), from = g.at(-k);
+            auto at = [&](const pairs::Coord& a) {
+                pairs::Coord r;
+                r.c2 = __shfl_sync(WHG_FULL_MASK, a.c2, to);
+                r.c1 = __shfl_sync(WHG_FULL_MASK, a.c1, to);
+                r.c0 = __shfl_sync(WHG_FULL_MASK, a.c0, to);
+                return r;
+            };
+            const pairs::Separation s = pairs::separation(pairs::difference(at(X), X), pairs::difference(at(Y), Y),
+                                                          pairs::difference(at(Z), Z));
+            const pairs::Pair r3 = pairs::inverse_cube(s);
+            const pairs::Pair wj = pairs::product(c.hmj[k - 1], r3);
+            bool fit = accept(s, wj.h, vl);
+            const pairs::Pair fx = pairs::product(wj, s.x), fy = pairs::product(wj, s.y), fz = pairs::product(wj, s.z);
+            pairs::accumulate(ax, fx.h, fx.l);
+            pairs::accumulate(ay, fy.h, fy.l);
+            pairs::accumulate(az, fz.h, fz.l);
+            if (2 * k < L) {                             // reaction on the partner: -hm_i (Q_j - Q_i)/r^3
+                const pairs::Pair wi = pairs::product(c.hmp, r3);
+                const float vj = __shfl_sync(WHG_FULL_MASK, vl, to);   // (every lane takes part)
+                fit = fit && accept(s, wi.h, vj);
+                const pairs::Pair gx = pairs::product(wi, s.x), gy = pairs::product(wi, s.y),
+                                  gz = pairs::product(wi, s.z);
+                auto take = [&](pairs::Pair& a, const pairs::Pair& f) {
+                    const float h = __shfl_sync(WHG_FULL_MASK, f.h, from), l = __shfl_sync(WHG_FULL_MASK, f.l, from);
+                    pairs::accumulate(a, -h, -l);
+                };
+                take(ax, gx);
+                take(ay, gy);
+                take(az, gz);
+            }
+            const bool on = (c.pairs_on >> k) & 1u;
+            ok = ok && (fit || !on);
+            if (hill) {
+                const double r2 = pairs::widen(s.r2, -K2);       // by the leading part, where that decides
+                const long long t = __double_as_longlong(thr2[k - 1]), b = __double_as_longlong(r2);
+                if (on && b - (1LL << 32) < t) close |= __double_as_longlong(r2 + pairs::widen(s.r2l, -K2)) < t;
+            }
+        }
+        if (GRM != 0) {
+            // a_GR(Q) = -6 (G m0)^2 Q / (c^2 |Q|^4); kgr = -6 m0^2 dt / c^2.
+            const pairs::Separation s = pairs::separation(pairs::own(X), pairs::own(Y), pairs::own(Z));
+            const float sc = fixed::bits_to_f32((unsigned)(127 + 1040 - eq) << 23);
+            pairs::Pair k;
+            k.h = pairs::mul(c.kgp.h, sc);
+            k.l = pairs::mul(c.kgp.l, sc);
+            const pairs::Pair w = pairs::product(k, pairs::inverse_fourth(s));
+            ok = ok && accept(s, -w.h, vl);
+            pairs::Pair fx = pairs::product(w, s.x), fy = pairs::product(w, s.y), fz = pairs::product(w, s.z);
+            if (GRM == 2) {                              // minus the mass-weighted sum, on every planet
+                const float mr = (float)c.mrat;
+                float bx = pairs::mul(mr, fx.h), by = pairs::mul(mr, fy.h), bz = pairs::mul(mr, fz.h);
+                sum_floats<L>(g, bx, by, bz);
+                if (L == 4 || L == 8) {
+                    const float b = bx;
+                    bx = __shfl_sync(WHG_FULL_MASK, b, g.base);
+                    by = __shfl_sync(WHG_FULL_MASK, b, g.base + L / 4);
+                    bz = __shfl_sync(WHG_FULL_MASK, b, g.base + L / 2);
+                }
+                pairs::accumulate(fx, -bx, 0.0f);
+                pairs::accumulate(fy, -by, 0.0f);
+                pairs::accumulate(fz, -bz, 0.0f);
+            }
+            pairs::accumulate(ax, fx.h, fx.l);
+            pairs::accumulate(ay, fy.h, fy.l);
+            pairs::accumulate(az, fz.h, fz.l);
+            const float mf = (float)c.m;
+            float px = pairs::mul(mf, fx.h), py = pairs::mul(mf, fy.h), pz = pairs::mul(mf, fz.h);
+            sum_floats<L>(g, px, py, pz);
+            double Px, Py, Pz;                           // the second jump
+            if (L == 4 || L == 8) {
+                gather3<L>(g, P.k + pairs::widen(px, K2), Px, Py, Pz);
+            } else {
+                Px = P.x + pairs::widen(px, K2);
+                Py = P.y + pairs::widen(py, K2);
+                Pz = P.z + pairs::widen(pz, K2);
+            }
+            qx = fma(c.jc, Px, qx);
+            qy = fma(c.jc, Py, qy);
+            qz = fma(c.jc, Pz, qz);
+        }
+        vx += pairs::widen(ax.h, K2) + pairs::widen(ax.l, K2);
+        vy += pairs::widen(ay.h, K2) + pairs::widen(ay.l, K2);
+        vz += pairs::widen(az.h, K2) + pairs::widen(az.l, K2);
+    }
+    if (GRM == 0 && !c.merged) {
+        qx = fma(c.jc, P.x, qx);
+        qy = fma(c.jc, P.y, qy);
+        qz = fma(c.jc, P.z, qz);
+    }
+    return ok;
+}
+
+// The sub-step: with float pairs, and in FP64 for the systems where that does
+// not hold (warp-uniform branch, per-system choice; it depends on the system's
+// state alone).  live: the lane's system is running (others are not redone).
+// q2, if Q2: the position during the kick.  Returns the close-encounter flag.
+template <int L, int GRM, bool Q2>
+__device__ __forceinline__ bool interact(const Group<L>& g, const Masses<L>& c, bool live, double& qx, double& qy,
+                                         double& qz, double& vx, double& vy, double& vz, const double* thr2,
+                                         bool hill, double* q2)
+{
+    bool close = false, ok = false;
+    double fqx = qx, fqy = qy, fqz = qz, fvx = vx, fvy = vy, fvz = vz;
+    if (!c.full) ok = interact_pairs<L, GRM, Q2>(g, c, fqx, fqy, fqz, fvx, fvy, fvz, thr2, hill, close, q2);
+    const unsigned redo = __ballot_sync(WHG_FULL_MASK, c.real && live && !ok);
+    if (redo) {
+        SubStep r{c.m, c.hm, c.mrat, c.jc, c.kgr, qx, qy, qz, vx, vy, vz, {0.0, 0.0, 0.0},
+                  {thr2[0], thr2[1], thr2[2], thr2[3]}, c.full, c.merged, false};
+        interact_general<L, GRM>(&r);
+        if (redo & g.mask()) {
+            fqx = r.qx; fqy = r.qy; fqz = r.qz;
+            fvx = r.vx; fvy = r.vy; fvz = r.vz;
+            close = r.close;
+            if (Q2) {
+                q2[0] = r.q2[0]; q2[1] = r.q2[1]; q2[2] = r.q2[2];
+            }
+        }
+    }
+    qx = fqx; qy = fqy; qz = fqz;
+    vx = fvx; vy = fvy; vz = fvz;
     return close;
 }
 
@@ -886,11 +1139,8 @@ __device__ __forceinline__ void step_body(const WhgState& st, const WhgBuckets& 
     const double rej2 = pl.has_sys ? st.rej2[s] : 0.0;
     const bool real = pl.has_sys && g.p < npl;
     bool alive = pl.has_sys && status == 0;
-    const double hm = dt * m;
-    const double jc = (0.5 * dt) / mu;
-    const double mrat = m / mu;
-    const double kgr = GRM ? (-6.0 * mu * mu * dt) / (st.c_light * st.c_light) : 0.0;
-    const bool full = st.full_rotation != 0;
+    const Masses<L> mc = masses_of<L, GRM>(g, real, m, mu, dt, st.c_light, GRM == 0 && st.merge, st.full_rotation != 0);
+    const bool hill = st.hill > 0.0;
     // close-encounter distances of this lane's pairs (once per launch)
     double thr2[4] = {0.0, 0.0, 0.0, 0.0};
     {
@@ -900,7 +1150,7 @@ __device__ __forceinline__ void step_body(const WhgState& st, const WhgBuckets& 
             const int to = g.at(k);
             const double mj = __shfl_sync(WHG_FULL_MASK, m, to);
             const double aj = __shfl_sync(WHG_FULL_MASK, a, to);
-            if (st.hill > 0.0 && k - 1 < 4) {
+            if (hill && k - 1 < 4) {
                 const double rh = st.hill * cbrt((m + mj) / (3.0 * mu)) * 0.5 * (a + aj);
                 thr2[k - 1] = rh * rh;
             }
@@ -914,16 +1164,8 @@ __device__ __forceinline__ void step_body(const WhgState& st, const WhgBuckets& 
         const double hK = (nstep0 + done == 0) ? 0.5 * dt : dt;
         const double r0sq = fma(qx, qx, fma(qy, qy, qz * qz));
         const bool far = __double_as_longlong(r0sq) > __double_as_longlong(rej2);
-        const bool bound = kepler_drift<NT>(mu, hK, qx, qy, qz, vx, vy, vz);
-        bool close;
-        if (GRM == 0 && st.merge) {                   // J(dt) I(dt): J and I commute without GR
-            jump<L>(g, m, 2.0 * jc, vx, vy, vz, qx, qy, qz);
-            close = kick<L, GRM>(g, qx, qy, qz, hm, mrat, kgr, thr2, vx, vy, vz, full);
-        } else {
-            jump<L>(g, m, jc, vx, vy, vz, qx, qy, qz);
-            close = kick<L, GRM>(g, qx, qy, qz, hm, mrat, kgr, thr2, vx, vy, vz, full);
-            jump<L>(g, m, jc, vx, vy, vz, qx, qy, qz);
-        }
+        const bool bound = kepler_drift<NT>(mu, hK, qx, qy, qz, vx, vy, vz, nullptr, alive);
+        const bool close = interact<L, GRM, false>(g, mc, alive, qx, qy, qz, vx, vy, vz, thr2, hill, nullptr);
         const bool fin = is_finite(qx) & is_finite(qy) & is_finite(qz) & is_finite(vx) &
                          is_finite(vy) & is_finite(vz);
         const unsigned bad_h = __ballot_sync(WHG_FULL_MASK, real && !bound) & gmask;
@@ -1109,7 +1351,7 @@ __device__ __forceinline__ int bucket_of(const WhgBuckets& bk, int w)
     }
 
 template <int NT, int GRM>
-__global__ void __launch_bounds__(WHG_MAX_BLOCK) k_step(WhgState st, WhgBuckets bk, long long n)
+__global__ void __launch_bounds__(WHG_MAX_BLOCK, WHG_STEP_BLOCKS) k_step(WhgState st, WhgBuckets bk, long long n)
 {
     const int w = warp_index();
     if (w >= bk.warp0[bk.nb]) return;                // whole warps beyond the last bucket
@@ -1149,7 +1391,7 @@ __device__ __noinline__ void queue_unit(const WhgState& st, const WhgBuckets& bk
 }
 
 template <int NT, int GRM>
-__global__ void __launch_bounds__(WHG_MAX_BLOCK) k_step_queue(WhgState st, WhgBuckets bk, long long n,
+__global__ void __launch_bounds__(WHG_MAX_BLOCK, WHG_STEP_BLOCKS) k_step_queue(WhgState st, WhgBuckets bk, long long n,
                                                              WhgQueue q)
 {
     const int G = bk.warp0[bk.nb];

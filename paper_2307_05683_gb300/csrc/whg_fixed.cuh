@@ -127,6 +127,20 @@ inline u64 umulhi64(u64 a, u64 b) { return (u64)(((unsigned __int128)a * b) >> 6
 inline float rsqrt_f32(float x) { return 1.0f / sqrtf(x); }
 #endif
 
+// Float operations that are never contracted: every kernel that inlines this
+// code computes the same bits.
+#if defined(__CUDA_ARCH__)
+__device__ __forceinline__ float add(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float sub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float mul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+#else
+inline float add(float a, float b) { volatile float r = a + b; return r; }
+inline float sub(float a, float b) { volatile float r = a - b; return r; }
+inline float mul(float a, float b) { volatile float r = a * b; return r; }
+inline float fma(float a, float b, float c) { return fmaf(a, b, c); }
+#endif
+
 // High word of a b, a, b < 2^63, to about one unit: the product of the low
 // words is left out (1/4 unit on average) and the rest truncated (1/2), and
 // K 2^-32 units are added so that the error's mean is zero (default 3/4).
@@ -172,7 +186,7 @@ WHG_HD u64 rsqrt62(u64 bits, int ef, int& half)
     const int ex = ef - 1023, odd = ex & 1;
     half = (ex - odd) / 2;
     const float mant = bits_to_f32(((u32)(127 + odd) << 23) | ((hi & 0x000fffffu) << 3) | (lo >> 29));
-    const u32 My = f32_to_u32(rsqrt_f32(mant) * 16777216.0f);            // 2^24 y, in [2^23, 2^24]
+    const u32 My = f32_to_u32(mul(rsqrt_f32(mant), 16777216.0f));            // 2^24 y, in [2^23, 2^24]
     const u64 S = (u64)My * My;                                          // y^2 in Q48
     const u64 Mx = ((u64)((hi & 0x000fffffu) | 0x00100000u) << 32) | lo; // mant 2^(52 - odd)
     const u64 plo = Mx * S, phi = umulhi64(Mx, S);                       // mant y^2 in Q(100 - odd)
@@ -182,6 +196,14 @@ WHG_HD u64 rsqrt62(u64 bits, int ef, int& half)
     const i64 Eh = (i32)hi32((u64)E);                                    // e 2^51
     const i64 U = (E >> 1) + 3 * ((Eh * Eh) >> 22);                      // (e/2 + 3 e^2/8) 2^83
     return ((u64)My << 38) + (u64)(((i64)My * (U >> 22) + 0xA00000) >> 23);   // (+: mean of both shifts' loss)
+}
+
+// A double as an integer on a grid: its significand (leading one at bit 62)
+// shifted right by sh (truncated; 0 from 63 on), with the sign.
+WHG_HD i64 to_fixed(u64 bits, int sh)
+{
+    const u64 m = significand62(bits) >> (sh > 63 ? 63 : sh);
+    return (i64)(bits >> 63 ? 0ull - m : m);
 }
 
 // Series coefficients 4^k/n! as round(4^k 2^q / n!), from an exact division.
@@ -230,27 +252,27 @@ WHG_HD void stumpff(u64 x, u64& c2, u64& c3)
 // Two Halley steps in FP32 for phi(s) = 0.
 WHG_HD float start(float a, float b, float B)
 {
-    float s = 1.0f + 0.5f * (a * a - a) - (1.0f / 6.0f) * b;
+    float s = fma(-1.0f / 6.0f, b, fma(0.5f, fma(a, a, -a), 1.0f));
     s = s < 0.6f ? 0.6f : (s > 1.7f ? 1.7f : s);
 #if defined(__CUDA_ARCH__)
 #pragma unroll
 #endif
     for (int it = 0; it < 2; ++it) {
-        const float u = s * s, z = B * u;
+        const float u = mul(s, s), z = mul(-B, u);
         float c2 = (float)(1.0 / 3628800.0), c3 = (float)(1.0 / 39916800.0);
-        c2 = (float)(1.0 / 40320.0) - z * c2;
-        c3 = (float)(1.0 / 362880.0) - z * c3;
-        c2 = (float)(1.0 / 720.0) - z * c2;
-        c3 = (float)(1.0 / 5040.0) - z * c3;
-        c2 = (float)(1.0 / 24.0) - z * c2;
-        c3 = (float)(1.0 / 120.0) - z * c3;
-        c2 = 0.5f - z * c2;
-        c3 = (float)(1.0 / 6.0) - z * c3;
-        const float g2 = u * c2, g3 = s * u * c3, g1 = s - B * g3, g0 = 1.0f - B * g2;
-        const float F = (s - 1.0f) + (a * g2 + b * g3);
-        const float R = 1.0f + (a * g1 + b * g2);
-        const float R1 = a * g0 + b * g1;
-        s = s - F * R * rcp_f32(R * R - 0.5f * F * R1);
+        c2 = fma(z, c2, (float)(1.0 / 40320.0));
+        c3 = fma(z, c3, (float)(1.0 / 362880.0));
+        c2 = fma(z, c2, (float)(1.0 / 720.0));
+        c3 = fma(z, c3, (float)(1.0 / 5040.0));
+        c2 = fma(z, c2, (float)(1.0 / 24.0));
+        c3 = fma(z, c3, (float)(1.0 / 120.0));
+        c2 = fma(z, c2, 0.5f);
+        c3 = fma(z, c3, (float)(1.0 / 6.0));
+        const float g2 = mul(u, c2), g3 = mul(mul(s, u), c3), g1 = fma(-B, g3, s), g0 = fma(-B, g2, 1.0f);
+        const float F = add(sub(s, 1.0f), fma(a, g2, mul(b, g3)));
+        const float R = fma(a, g1, fma(b, g2, 1.0f));
+        const float R1 = fma(a, g0, mul(b, g1));
+        s = fma(-mul(F, R), rcp_f32(fma(R, R, mul(-0.5f, mul(F, R1)))), s);
     }
     return s;
 }
@@ -320,13 +342,13 @@ WHG_HD bool solve(double mu, double h, double r0sq, double eta0, double v2, Solu
     i64 Bs = (i64)(2 * mq - Vq);                                         // Q61
     Bs = Bs < 0 ? 0 : Bs;
     const u64 B = (u64)Bs << 1;                                          // Q62
-    const float af = (neg ? -1.0f : 1.0f) * (u32_to_f32(hi32(amag)) * (1.0f / 1073741824.0f));
-    const float bf = u32_to_f32(hi32(b2)) * (1.0f / 536870912.0f) - 2.0f;
-    const float Bf = u32_to_f32(hi32((u64)Bs)) * (1.0f / 536870912.0f);
+    const float am = mul(u32_to_f32(hi32(amag)), 1.0f / 1073741824.0f), af = neg ? -am : am;
+    const float bf = fma(u32_to_f32(hi32(b2)), 1.0f / 536870912.0f, -2.0f);
+    const float Bf = mul(u32_to_f32(hi32((u64)Bs)), 1.0f / 536870912.0f);
     if (!(amag < one62 - (one62 >> 10) && bf < 1.999f && bf > -1.999f && Bf < 1.999f)) return false;
     const float sf = start(af, bf, Bf);
-    if (!(sf > 0.5625f && sf < 1.75f && Bf * (sf * sf) < 1.99f)) return false;
-    const u32 sh = f32_to_u32(sf * 1073741824.0f) - 724u;                // Q30, 2^-20.5 low
+    if (!(sf > 0.5625f && sf < 1.75f && mul(Bf, mul(sf, sf)) < 1.99f)) return false;
+    const u32 sh = f32_to_u32(mul(sf, 1073741824.0f)) - 724u;                // Q30, 2^-20.5 low
 
     // series and g_n at the start
     const u64 u = (u64)sh * sh;                                          // s^2, Q60
@@ -346,7 +368,7 @@ WHG_HD bool solve(double mu, double h, double r0sq, double eta0, double v2, Solu
         return false;
 
     // 1/R to ~2^-44: FP32 seed and one Newton correction
-    const u32 y0 = f32_to_u32(rcp_f32(u32_to_f32((u32)(R >> 29))) * 72057594037927936.0f);   // Q25
+    const u32 y0 = f32_to_u32(mul(rcp_f32(u32_to_f32((u32)(R >> 29))), 72057594037927936.0f));   // Q25
     const i64 D = (i64)(0ull - R * (u64)y0);                             // (1 - R y0) 2^85
     const u64 y = ((u64)y0 << 37) + (u64)(((i64)(i32)y0 * (i64)(i32)(D >> 32)) >> 16);       // Q62
 
@@ -370,7 +392,7 @@ WHG_HD bool solve(double mu, double h, double r0sq, double eta0, double v2, Solu
     const i64 d1 = (i64)(one60 - mulhi(Rn << 2, y));                     // Q60
     if (!(d1 < (1ll << 40) && d1 > -(1ll << 40))) return false;
     const i64 e1 = d1 >> 13;                                             // Q47
-    const i64 t = d1 + (i64)(((u64)(e1 * e1)) >> 34);                    // Q60
+    const i64 t = d1 + (((i64)(i32)e1 * (i32)e1) >> 34);                    // Q60
     const u64 yn = y + mulhi((u64)((t << 4) + (1ll << 48)), y) - (y >> 16);                  // Q62
 
     const u64 mg3 = mulhi(mq, G3 << 2);                                  // Q60
