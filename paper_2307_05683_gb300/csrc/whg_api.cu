@@ -123,14 +123,13 @@ int warps_capacity(int S, int Nmax, int Lfixed)
 }
 
 // Bucket systems by lanes per system.  nplan may be null (all Nmax planets).
-// perm receives, for every internal system, the caller's index (the
-// identity when every system gets the same lane group, which repacking
-// starts from); returns false when the layout is the identity.
-bool plan_layout(int S, int Nmax, int Lfixed, const int* nplan, WhgBuckets* bk, int* perm)
+// perm receives, for every internal system, the caller's index; it stays empty
+// when every system gets the same lane group, where the layout is the
+// identity.  Returns false when it is.
+bool plan_layout(int S, int Nmax, int Lfixed, const int* nplan, WhgBuckets* bk, std::vector<int>& perm)
 {
     *bk = WhgBuckets{};
     if (Lfixed || !nplan) {
-        for (int s = 0; s < S; ++s) perm[s] = s;
         const int L = Lfixed ? Lfixed : whg_lanes_for_planets(Nmax);
         bk->nb = 1;
         bk->L[0] = L;
@@ -161,6 +160,7 @@ bool plan_layout(int S, int Nmax, int Lfixed, const int* nplan, WhgBuckets* bk, 
     bk->warp0[nb] = warps;
     bk->sys0[nb] = S;
     bool identity = true;
+    perm.resize((size_t)S);
     for (int s = 0; s < S; ++s) {
         const int i = next[lanes_of(s)]++;
         perm[i] = s;
@@ -458,11 +458,15 @@ int whg_set_stream(whg_ctx* c, void* cuda_stream)
 // host, or null) and run the init kernel on the inputs `in`.
 static int init_common(whg_ctx* c, const WhgIn& in, const int* nplan_host)
 {
-    std::vector<int> perm((size_t)c->S);
-    const bool permuted = plan_layout(c->S, c->Nmax, c->Lfixed, nplan_host, &c->bk, perm.data());
+    std::vector<int> perm;
+    const bool permuted = plan_layout(c->S, c->Nmax, c->Lfixed, nplan_host, &c->bk, perm);
     if (c->bk.warp0[c->bk.nb] > c->warps_cap)
         return fail(c, WHG_EINVAL, "internal layout exceeds capacity");
     if (permuted || c->repack_buf) {                     // repacking needs the map even if identity
+        if (perm.empty()) {
+            perm.resize((size_t)c->S);
+            for (int s = 0; s < c->S; ++s) perm[(size_t)s] = s;
+        }
         WHG_CUDA(c, cudaMemcpyAsync(c->perm_d, perm.data(), perm.size() * sizeof(int),
                                     cudaMemcpyHostToDevice, c->stream));
         c->st.perm = c->perm_d;

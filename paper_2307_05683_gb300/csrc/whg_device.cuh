@@ -1015,97 +1015,152 @@ __device__ __forceinline__ int user_index(const WhgState& st, int sys)
 // Kernel bodies.  A warp belongs to one bucket; shuffles use the full warp
 // mask, so no lane leaves a body before its last shuffle.
 
+// The quotients x[0..2]/a and x[3..5]/b in every lane of the system, each taken
+// by one lane (an FP64 division is about ten FP64 instructions).
+template <int L>
+__device__ __forceinline__ void group_divide6(const Group<L>& g, const double* x, double a, double b, double* q)
+{
+    constexpr int kRounds = (6 + L - 1) / L;
+    double mine[kRounds];
+#pragma unroll
+    for (int r = 0; r < kRounds; ++r) {
+        double n = 0.0, d = a;
+#pragma unroll
+        for (int p = 0; p < L; ++p) {
+            const int j = r * L + p;
+            if (j < 6 && g.p == p) {
+                n = x[j];
+                d = j < 3 ? a : b;
+            }
+        }
+        mine[r] = n / d;
+    }
+#pragma unroll
+    for (int j = 0; j < 6; ++j) q[j] = __shfl_sync(WHG_FULL_MASK, mine[j / L], g.in_group ? g.base + j % L : g.lane);
+}
+
+// Sums over the system's lanes of seven values, the same bits in every lane.
+// L = 8: reduce-scatter by xor partners (4 + 2 + 1 additions instead of 21).
+template <int L>
+__device__ __forceinline__ void group_sum7(const Group<L>& g, double* x)
+{
+    if (L == 8) {
+        double v[8] = {x[0], x[1], x[2], x[3], x[4], x[5], x[6], 0.0};
+#pragma unroll
+        for (int o = 4; o; o >>= 1) {
+            const bool hi = (g.p & o) != 0;      // keeps the upper o values
+#pragma unroll
+            for (int j = 0; j < o; ++j) {
+                const double keep = hi ? v[j + o] : v[j], send = hi ? v[j] : v[j + o];
+                v[j] = keep + __shfl_xor_sync(WHG_FULL_MASK, send, o);
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < 7; ++j) x[j] = __shfl_sync(WHG_FULL_MASK, v[0], g.base + j);
+    } else {
+#pragma unroll
+        for (int j = 0; j < 7; ++j) x[j] = group_sum<L>(g, x[j]);
+    }
+}
+
 // Inertial -> DH (Sec. 3.1): Q_i = x_i - x_0, v_i = u_i - V_cm; M, X_cm, V_cm
-// kept; initial osculating a_i (mu = G(m0 + m_i)) for the stop rules.
+// kept; initial osculating a_i (mu = G(m0 + m_i)) for the stop rules, when one
+// is on.  Each lane checks and converts its own planet (and the star); the
+// sums are over lanes, and the divisions by M one per lane.  (With every lane
+// summing all bodies: 2^20 8-planet systems took 6.6 ms, one system 24 us.)
 template <int L>
 __device__ __forceinline__ void init_body(const WhgState& st, const WhgBuckets& bk, const WhgIn& in,
                                           int b, int w)
 {
     const Place<L> pl(st, bk, b, w);
-    const int p = pl.g.p;
+    const Group<L>& g = pl.g;
+    const int p = g.p;
     const size_t lane = pl.lane;
-    int n = 0, ok = 0;
-    double M = 0.0, xc[3] = {0.0, 0.0, 0.0}, vc[3] = {0.0, 0.0, 0.0}, m0 = 1.0, dt = 1.0e-3;
-    double amax = 0.0, a_mine = 0.0;
+    int n = 0;
+    double m0 = 1.0, dt = 1.0e-3, m = 0.0, a = 0.0;
+    double x0[3] = {0.0, 0.0, 0.0}, u0[3] = {0.0, 0.0, 0.0}, x[3] = {0.0, 0.0, 0.0}, u[3] = {0.0, 0.0, 0.0};
+    bool head = false, mine = true;              // the system's own values; this lane's bodies
     if (pl.has_sys) {
-        const int u = user_index(st, pl.sys);
+        const int us = user_index(st, pl.sys);
         const int B = 1 + st.Nmax;
-        const double* ms = in.masses + (size_t)u * B;
-        const double* xs = in.pos + (size_t)u * B * 3;
-        const double* us = in.vel + (size_t)u * B * 3;
-        n = in.nplan ? in.nplan[u] : st.Nmax;
-        dt = in.dt[u];
+        const double* ms = in.masses + (size_t)us * B;
+        const double* xs = in.pos + (size_t)us * B * 3;
+        const double* vs = in.vel + (size_t)us * B * 3;
+        n = in.nplan ? in.nplan[us] : st.Nmax;
+        dt = in.dt[us];
         m0 = ms[0];
-        ok = n >= 1 && n <= st.Nmax && n <= L && dt > 0.0 && is_finite(dt) && m0 > 0.0 &&
-             is_finite(m0);
-        if (ok) {
-            for (int k = 0; k <= n; ++k) {
-                M += ms[k];
-                ok &= ms[k] >= 0.0 && is_finite(ms[k]);
-                for (int c = 0; c < 3; ++c) {
-                    ok &= is_finite(xs[3 * k + c]) && is_finite(us[3 * k + c]);
-                    xc[c] += ms[k] * xs[3 * k + c];
-                    vc[c] += ms[k] * us[3 * k + c];
-                }
-                if (k > 0) {
-                    ok &= !(xs[3 * k] == xs[0] && xs[3 * k + 1] == xs[1] && xs[3 * k + 2] == xs[2]);
-                    double r2 = 0.0, w2 = 0.0;
-                    for (int c = 0; c < 3; ++c) {
-                        const double dx = __dsub_rn(xs[3 * k + c], xs[c]);
-                        const double du = __dsub_rn(us[3 * k + c], us[c]);
-                        r2 = __dadd_rn(r2, __dmul_rn(dx, dx));
-                        w2 = __dadd_rn(w2, __dmul_rn(du, du));
-                    }
-                    const double a = 1.0 / __dsub_rn(2.0 / sqrt(r2), w2 / __dadd_rn(m0, ms[k]));
-                    amax = fmax(amax, a);
-                    if (k == p + 1) a_mine = a;
-                }
-            }
-            for (int c = 0; c < 3; ++c) {
-                xc[c] /= M;
-                vc[c] /= M;
-            }
-        }
-        if (ok && p < n) {
-            st.m[lane] = ms[1 + p];
-            st.qx[lane] = xs[3 * (1 + p) + 0] - xs[0];
-            st.qy[lane] = xs[3 * (1 + p) + 1] - xs[1];
-            st.qz[lane] = xs[3 * (1 + p) + 2] - xs[2];
-            st.vx[lane] = us[3 * (1 + p) + 0] - vc[0];
-            st.vy[lane] = us[3 * (1 + p) + 1] - vc[1];
-            st.vz[lane] = us[3 * (1 + p) + 2] - vc[2];
-            st.a0[lane] = a_mine;
-        }
-    }
-    if (!(ok && p < n)) {                            // no planet on this lane
-        st.m[lane] = 0.0;
-        st.qx[lane] = parked_x(p);
-        st.qy[lane] = 0.0;
-        st.qz[lane] = 0.0;
-        st.vx[lane] = 0.0;
-        st.vy[lane] = 0.0;
-        st.vz[lane] = 0.0;
-        st.a0[lane] = 0.0;
-    }
-    if (pl.has_sys && p == 0) {
-        const int s = pl.sys;
-        if (!ok) {
-            m0 = 1.0;
-            dt = 1.0e-3;
-            M = 1.0;
-        }
-        st.m0[s] = m0;
-        st.dt[s] = dt;
-        st.M[s] = M;
+        head = n >= 1 && n <= st.Nmax && n <= L && dt > 0.0 && is_finite(dt) && m0 > 0.0 && is_finite(m0);
+#pragma unroll
         for (int c = 0; c < 3; ++c) {
-            st.xcm[(size_t)c * st.S + s] = xc[c];
-            st.vcm[(size_t)c * st.S + s] = vc[c];
+            x0[c] = xs[c];
+            u0[c] = vs[c];
+            mine = mine && is_finite(x0[c]) && is_finite(u0[c]);
+        }
+        if (head && p < n) {
+            m = ms[1 + p];
+            mine = mine && m >= 0.0 && is_finite(m);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                x[c] = xs[3 * (1 + p) + c];
+                u[c] = vs[3 * (1 + p) + c];
+                mine = mine && is_finite(x[c]) && is_finite(u[c]);
+            }
+            mine = mine && !(x[0] == x0[0] && x[1] == x0[1] && x[2] == x0[2]);
+            if (st.hill > 0.0 || st.eject > 0.0) {
+                double r2 = 0.0, w2 = 0.0;
+                for (int c = 0; c < 3; ++c) {
+                    const double dx = __dsub_rn(x[c], x0[c]);
+                    const double du = __dsub_rn(u[c], u0[c]);
+                    r2 = __dadd_rn(r2, __dmul_rn(dx, dx));
+                    w2 = __dadd_rn(w2, __dmul_rn(du, du));
+                }
+                a = 1.0 / __dsub_rn(2.0 / sqrt(r2), w2 / __dadd_rn(m0, m));
+            }
+        }
+    }
+    const unsigned bad = __ballot_sync(WHG_FULL_MASK, !mine) & g.mask();
+    const bool ok = head && bad == 0u;
+    double s[7] = {m, m * x[0], m * x[1], m * x[2], m * u[0], m * u[1], m * u[2]};
+    if (p == 0) {                                // with the star
+        s[0] += m0;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            s[1 + c] = fma(m0, x0[c], s[1 + c]);
+            s[4 + c] = fma(m0, u0[c], s[4 + c]);
+        }
+    }
+    group_sum7<L>(g, s);
+    double cm[6];                                // X_cm, V_cm
+    group_divide6<L>(g, s + 1, s[0], s[0], cm);
+    double amax = 0.0;
+    if (st.eject > 0.0) {
+        amax = fmax(0.0, a);                     // (a NaN counts as 0)
+#pragma unroll
+        for (int k = 1; k < L; ++k) amax = fmax(amax, __shfl_sync(WHG_FULL_MASK, a, g.at(k)));
+    }
+    const bool live = ok && p < n;
+    st.m[lane] = live ? m : 0.0;
+    st.qx[lane] = live ? x[0] - x0[0] : parked_x(p);
+    st.qy[lane] = live ? x[1] - x0[1] : 0.0;
+    st.qz[lane] = live ? x[2] - x0[2] : 0.0;
+    st.vx[lane] = live ? u[0] - cm[3] : 0.0;
+    st.vy[lane] = live ? u[1] - cm[4] : 0.0;
+    st.vz[lane] = live ? u[2] - cm[5] : 0.0;
+    st.a0[lane] = live ? a : 0.0;
+    if (pl.has_sys && p == 0) {
+        const int i = pl.sys;
+        st.m0[i] = ok ? m0 : 1.0;
+        st.dt[i] = ok ? dt : 1.0e-3;
+        st.M[i] = ok ? s[0] : 1.0;
+        for (int c = 0; c < 3; ++c) {
+            st.xcm[(size_t)c * st.S + i] = ok ? cm[c] : 0.0;
+            st.vcm[(size_t)c * st.S + i] = ok ? cm[3 + c] : 0.0;
         }
         const double rej = st.eject * amax;
-        st.rej2[s] = (st.eject > 0.0 && ok && amax > 0.0) ? rej * rej : __longlong_as_double(0x7ff0000000000000LL);
-        st.nplan[s] = ok ? n : 0;
-        st.status[s] = ok ? 0 : WHG_STATUS_INVALID;
-        st.nstep[s] = 0;
+        st.rej2[i] = (st.eject > 0.0 && ok && amax > 0.0) ? rej * rej : __longlong_as_double(0x7ff0000000000000LL);
+        st.nplan[i] = ok ? n : 0;
+        st.status[i] = ok ? 0 : WHG_STATUS_INVALID;
+        st.nstep[i] = 0;
     }
 }
 
@@ -1212,21 +1267,22 @@ __device__ __forceinline__ void read_body(const WhgState& st, const WhgBuckets& 
     const double dt = pl.has_sys ? st.dt[s] : 1.0e-3;
     const long long ns = pl.has_sys ? st.nstep[s] : 0;
     if (ns > 0) kepler_drift<NT>(mu, 0.5 * dt, qx, qy, qz, vx, vy, vz);
-    const double sqx = group_sum<L>(g, m * qx), sqy = group_sum<L>(g, m * qy), sqz = group_sum<L>(g, m * qz);
-    const double spx = group_sum<L>(g, m * vx), spy = group_sum<L>(g, m * vy), spz = group_sum<L>(g, m * vz);
+    const MassSum SQ = mass_sum<L>(g, m, qx, qy, qz), SP = mass_sum<L>(g, m, vx, vy, vz);
+    const double sums[6] = {SQ.x, SQ.y, SQ.z, SP.x, SP.y, SP.z};
+    double cm[6];                                    // sum m Q / M, sum m v / m0
+    group_divide6<L>(g, sums, pl.has_sys ? st.M[s] : 1.0, mu, cm);
     if (!pl.has_sys) return;                         // after the last shuffle
     const int npl = st.nplan[s];
     const int u = user_index(st, s);
     const int B = 1 + st.Nmax;
     const double t = (double)ns * dt;
-    const double M = st.M[s];
-    const double sq[3] = {sqx, sqy, sqz}, sp[3] = {spx, spy, spz}, q[3] = {qx, qy, qz}, v[3] = {vx, vy, vz};
+    const double q[3] = {qx, qy, qz}, v[3] = {vx, vy, vz};
     double x0[3], u0[3], V[3];
     for (int c = 0; c < 3; ++c) {
         const double X = st.xcm[(size_t)c * st.S + s];
         V[c] = st.vcm[(size_t)c * st.S + s];
-        x0[c] = (X + V[c] * t) - sq[c] / M;
-        u0[c] = V[c] - sp[c] / mu;
+        x0[c] = (X + V[c] * t) - cm[c];
+        u0[c] = V[c] - cm[3 + c];
     }
     for (int slot = g.p; slot < st.Nmax; slot += L) {    // planet slots of this lane
         const size_t o = ((size_t)u * B + 1 + slot) * 3;
@@ -1263,21 +1319,23 @@ __device__ __forceinline__ void energy_body(const WhgState& st, const WhgBuckets
     const double dt = pl.has_sys ? st.dt[s] : 1.0e-3;
     if (pl.has_sys && st.nstep[s] > 0)
         kepler_drift<NT>(mu, 0.5 * dt, qx, qy, qz, vx, vy, vz);
-    const double r2 = fma(qx, qx, fma(qy, qy, qz * qz));
-    double pair = 0.0;
+    const double ri = rsqrt(fma(qx, qx, fma(qy, qy, qz * qz)));
+    double pair = 0.0;                               // each pair once: distance L/2 by halves in both lanes
 #pragma unroll
-    for (int k = 1; k < L; ++k) {
+    for (int k = 1; 2 * k <= L; ++k) {
         const int j = g.at(k);
         const double dx = __shfl_sync(WHG_FULL_MASK, qx, j) - qx;
         const double dy = __shfl_sync(WHG_FULL_MASK, qy, j) - qy;
         const double dz = __shfl_sync(WHG_FULL_MASK, qz, j) - qz;
         const double mj = __shfl_sync(WHG_FULL_MASK, m, j);
-        pair += m * mj / sqrt(fma(dx, dx, fma(dy, dy, dz * dz)));
+        const double e = (m * mj) * rsqrt(fma(dx, dx, fma(dy, dy, dz * dz)));
+        pair += 2 * k == L ? 0.5 * e : e;
     }
-    double part = 0.5 * m * fma(vx, vx, fma(vy, vy, vz * vz)) - mu * m / sqrt(r2) - 0.5 * pair;
-    if (GRM != 0) part += -3.0 * m * mu * mu / (st.c_light * st.c_light * r2);
+    double part = 0.5 * m * fma(vx, vx, fma(vy, vy, vz * vz)) - mu * m * ri - pair;
+    if (GRM != 0) part -= (3.0 * m * mu * mu / (st.c_light * st.c_light)) * (ri * ri);
     const double tot = group_sum<L>(g, part);
-    const double px = group_sum<L>(g, m * vx), py = group_sum<L>(g, m * vy), pz = group_sum<L>(g, m * vz);
+    const MassSum P = mass_sum<L>(g, m, vx, vy, vz);
+    const double px = P.x, py = P.y, pz = P.z;
     if (!pl.has_sys || g.p != 0) return;
     double h0 = 0.0;
     for (int c = 0; c < 3; ++c) {
