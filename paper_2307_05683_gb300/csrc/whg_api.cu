@@ -244,7 +244,7 @@ constexpr long long kQueueSpinLimit = 1LL << 26;
 cudaError_t launch_steps(whg_ctx* c, long long n_steps, const WhgLaunch& l)
 {
     const long long qs = c->opt.queue_steps;
-    if (!c->q_next || n_steps < kQueueMinUnits * qs)
+    if (!c->q_next || n_steps < kQueueMinUnits * qs || whg_few_warps(c->bk))
         return whg_launch_step(c->st, c->bk, n_steps, c->opt.newton_terms, c->opt.gr_mode, l);
     WhgQueue q{c->q_next, c->q_done, c->q_err, qs, (int)((n_steps + qs - 1) / qs), kQueueSpinLimit};
     cudaError_t e = cudaMemsetAsync(c->q_next, 0, sizeof(unsigned long long), l.stream);

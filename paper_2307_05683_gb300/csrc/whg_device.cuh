@@ -32,12 +32,6 @@
 
 #define WHG_FULL_MASK 0xffffffffu
 
-// Blocks of WHG_MAX_BLOCK threads that the step kernels leave room for on an SM:
-// 2 (128 registers a thread, 16 resident warps) against 1 (160-186 registers,
-// 10-12 warps): 8192 8-planet systems 1.03e9 against 0.90e9 system-steps/s,
-// 65,536 1.15e9 against 1.09e9.
-#define WHG_STEP_BLOCKS 2
-
 namespace whg {
 
 // ------------------------------------------------------------------------
@@ -1408,8 +1402,12 @@ __device__ __forceinline__ int bucket_of(const WhgBuckets& bk, int w)
     default: { constexpr int L_ = 8; CALL; } break; \
     }
 
-template <int NT, int GRM>
-__global__ void __launch_bounds__(WHG_MAX_BLOCK, WHG_STEP_BLOCKS) k_step(WhgState st, WhgBuckets bk, long long n)
+// BLOCKS: blocks of WHG_MAX_BLOCK threads that the register count leaves room for
+// on an SM.  2 (128 registers, 16 resident one-warp blocks) where more than
+// 8 warps per SM share the pipes; 1 (any number of registers, a schedule for
+// one warp's own latency) below.
+template <int NT, int GRM, int BLOCKS>
+__global__ void __launch_bounds__(WHG_MAX_BLOCK, BLOCKS) k_step(WhgState st, WhgBuckets bk, long long n)
 {
     const int w = warp_index();
     if (w >= bk.warp0[bk.nb]) return;                // whole warps beyond the last bucket
@@ -1449,7 +1447,7 @@ __device__ __noinline__ void queue_unit(const WhgState& st, const WhgBuckets& bk
 }
 
 template <int NT, int GRM>
-__global__ void __launch_bounds__(WHG_MAX_BLOCK, WHG_STEP_BLOCKS) k_step_queue(WhgState st, WhgBuckets bk, long long n,
+__global__ void __launch_bounds__(WHG_MAX_BLOCK, 2) k_step_queue(WhgState st, WhgBuckets bk, long long n,
                                                              WhgQueue q)
 {
     const int G = bk.warp0[bk.nb];

@@ -137,6 +137,9 @@ cudaError_t whg_launch_repack(const WhgState& st, const WhgState& scratch, const
 cudaError_t whg_launch_raw(const WhgState&, const WhgBuckets&, const WhgOut&, int set, const WhgLaunch&);
 cudaError_t whg_launch_step(const WhgState&, const WhgBuckets&, long long nsteps, int newton_terms,
                             int gr_mode, const WhgLaunch&);
+// Whether an ensemble's warps leave every SM at most 8 of them: such launches run
+// the step kernel built for few warps, and have no use for the work queue.
+bool whg_few_warps(const WhgBuckets&);
 // Step kernel over the work queue (q.next and q.done zeroed by the caller).
 cudaError_t whg_launch_step_queue(const WhgState&, const WhgBuckets&, long long nsteps, int newton_terms,
                                   int gr_mode, const WhgQueue& q, cudaStream_t stream);
@@ -146,6 +149,8 @@ cudaError_t whg_launch_energy(const WhgState&, const WhgBuckets&, const WhgOut&,
                               int gr_mode, const WhgLaunch&);
 cudaError_t whg_launch_step_nt6(const WhgState&, const WhgBuckets&, long long, int, const WhgLaunch&);
 cudaError_t whg_launch_step_nt8(const WhgState&, const WhgBuckets&, long long, int, const WhgLaunch&);
+cudaError_t whg_launch_step_few_nt6(const WhgState&, const WhgBuckets&, long long, int, const WhgLaunch&);
+cudaError_t whg_launch_step_few_nt8(const WhgState&, const WhgBuckets&, long long, int, const WhgLaunch&);
 cudaError_t whg_launch_step_queue_nt6(const WhgState&, const WhgBuckets&, long long, int, const WhgQueue&,
                                       cudaStream_t);
 cudaError_t whg_launch_step_queue_nt8(const WhgState&, const WhgBuckets&, long long, int, const WhgQueue&,

@@ -154,9 +154,28 @@ cudaError_t whg_launch_raw(const WhgState& st, const WhgBuckets& bk, const WhgOu
     return cudaGetLastError();
 }
 
+// Up to 8 warps per SM (2 per sub-partition) a step is bound by each warp's own
+// chain of instructions, and the kernel with more registers is the faster one;
+// above, the resident warps count.  Measured, 8-planet systems, us per step, few /
+// many: 2432 systems (4 warps per SM) 4.21 / 4.76, 4096 (6.7) 4.82 / 5.33,
+// 8192 (13.5) 9.1 / 7.98.  Results are the same bits.
+bool whg_few_warps(const WhgBuckets& bk)
+{
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return bk.warp0[bk.nb] <= 8 * sms;
+}
+
 cudaError_t whg_launch_step(const WhgState& st, const WhgBuckets& bk, long long n, int newton_terms,
                             int gr_mode, const WhgLaunch& l)
 {
+    if (whg_few_warps(bk))
+        return newton_terms == 6 ? whg_launch_step_few_nt6(st, bk, n, gr_mode, l)
+                                 : whg_launch_step_few_nt8(st, bk, n, gr_mode, l);
     return newton_terms == 6 ? whg_launch_step_nt6(st, bk, n, gr_mode, l)
                              : whg_launch_step_nt8(st, bk, n, gr_mode, l);
 }

@@ -6,11 +6,11 @@ cudaError_t whg_launch_step_nt6(const WhgState& st, const WhgBuckets& bk, long l
                                   const WhgLaunch& l)
 {
     if (gr_mode == 0)
-        whg::k_step<6, 0><<<l.grid, l.block, 0, l.stream>>>(st, bk, n);
+        whg::k_step<6, 0, 2><<<l.grid, l.block, 0, l.stream>>>(st, bk, n);
     else if (gr_mode == 1)
-        whg::k_step<6, 1><<<l.grid, l.block, 0, l.stream>>>(st, bk, n);
+        whg::k_step<6, 1, 2><<<l.grid, l.block, 0, l.stream>>>(st, bk, n);
     else
-        whg::k_step<6, 2><<<l.grid, l.block, 0, l.stream>>>(st, bk, n);
+        whg::k_step<6, 2, 2><<<l.grid, l.block, 0, l.stream>>>(st, bk, n);
     return cudaGetLastError();
 }
 
