@@ -104,6 +104,7 @@ WhgLaunch launch_cfg(const whg_ctx* c)
     l.grid = (int)((threads + c->block - 1) / c->block);
     if (l.grid < 1) l.grid = 1;
     l.stream = c->stream;
+    l.sms = 0;
     return l;
 }
 
@@ -940,6 +941,7 @@ static WhgLaunch chain_cfg(const whg_ctx* c, bool on_split)
         l.grid = (int)((threads + 127) / 128);
         if (l.grid < 1) l.grid = 1;
         l.stream = c->s_chain;
+        l.sms = c->chain_sms;
     }
     return l;
 }

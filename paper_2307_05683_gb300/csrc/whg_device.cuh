@@ -844,10 +844,10 @@ __device__ __forceinline__ bool interact_pairs(const Group<L>& g, const Masses<L
         const pairs::Coord Y = pairs::chunks(fixed::to_fixed(by, 5 + eq - ey));
         const pairs::Coord Z = pairs::chunks(fixed::to_fixed(bz, 5 + eq - ez));
         pairs::Pair ax = {0.0f, 0.0f}, ay = {0.0f, 0.0f}, az = {0.0f, 0.0f};
-        // a term is accepted up to 2^-11 of the velocity, and weaker for
+        // a term is accepted up to 2^-10 of the velocity, and weaker for
         // separations where the grid shows (below 2^-7 of its extent)
         auto accept = [](const pairs::Separation& s, float w, float v) {
-            return fmaxf(pairs::mul(w, pairs::mul(s.r2, s.y1)), pairs::mul(w, 128.0f)) <= pairs::mul(v, 1.0f / 2048.0f);
+            return fmaxf(pairs::mul(w, pairs::mul(s.r2, s.y1)), pairs::mul(w, 256.0f)) <= pairs::mul(v, 1.0f / 1024.0f);
         };
 #pragma unroll
         for (int k = 1; 2 * k <= L; ++k) {

@@ -176,28 +176,6 @@ WHG_HD double to_double(u64 n, int s)
     return from_bits(r + ((u64)(u32)(1023 + 61 - lz - s) << 52));
 }
 
-// mant^(-1/2) in Q62, mant = x 4^-half in [1, 4), for a normal double x > 0
-// with exponent field ef.  FP32 seed y = My 2^-24, then y (1 + e/2 + 3 e^2/8)
-// with e = 1 - mant y^2 exact in 64-bit fixed point (|e| < 2^-21, so E = e 2^83
-// fits; the neglected e^3 is below 2^-62).
-WHG_HD u64 rsqrt62(u64 bits, int ef, int& half)
-{
-    const u32 hi = hi32(bits), lo = (u32)bits;
-    const int ex = ef - 1023, odd = ex & 1;
-    half = (ex - odd) / 2;
-    const float mant = bits_to_f32(((u32)(127 + odd) << 23) | ((hi & 0x000fffffu) << 3) | (lo >> 29));
-    const u32 My = f32_to_u32(mul(rsqrt_f32(mant), 16777216.0f));            // 2^24 y, in [2^23, 2^24]
-    const u64 S = (u64)My * My;                                          // y^2 in Q48
-    const u64 Mx = ((u64)((hi & 0x000fffffu) | 0x00100000u) << 32) | lo; // mant 2^(52 - odd)
-    const u64 plo = Mx * S, phi = umulhi64(Mx, S);                       // mant y^2 in Q(100 - odd)
-    const int sh = 17 - odd;                                             // to Q83
-    const u64 P83 = (plo >> sh) | (phi << (64 - sh));                    // mant y^2 mod 2^64 = -e 2^83
-    const i64 E = -(i64)P83;
-    const i64 Eh = (i32)hi32((u64)E);                                    // e 2^51
-    const i64 U = (E >> 1) + 3 * ((Eh * Eh) >> 22);                      // (e/2 + 3 e^2/8) 2^83
-    return ((u64)My << 38) + (u64)(((i64)My * (U >> 22) + 0xA00000) >> 23);   // (+: mean of both shifts' loss)
-}
-
 // A double as an integer on a grid: its significand (leading one at bit 62)
 // shifted right by sh (truncated; 0 from 63 on), with the sign.
 WHG_HD i64 to_fixed(u64 bits, int sh)
@@ -205,6 +183,11 @@ WHG_HD i64 to_fixed(u64 bits, int sh)
     const u64 m = significand62(bits) >> (sh > 63 ? 63 : sh);
     return (i64)(bits >> 63 ? 0ull - m : m);
 }
+
+WHG_HD int larger(int a, int b) { return a > b ? a : b; }
+
+// 2^k as a float, 0 below 2^-126 (k < 128).
+WHG_HD float power2(int k) { return bits_to_f32(k < -126 ? 0u : (u32)(k + 127) << 23); }
 
 // Series coefficients 4^k/n! as round(4^k 2^q / n!), from an exact division.
 constexpr u64 coef(int k, int n, int q)
@@ -308,44 +291,55 @@ WHG_HD bool solve(double mu, double h, double r0sq, double eta0, double v2, Solu
     // r0 within 2^+-100, h within 2^+-150, mu within 2^+-100 of one: every
     // result is a normal double; inf and NaN are outside.  (A zero or subnormal
     // eta0 or v^2 counts as 2^-1023, which its fixed-point form rounds to 0.)
-    if ((u32)(er - 823) > 400u || ee > 1623 || ev > 1623 || (u32)(eh - 873) > 300u || (u32)(emu - 923) > 200u)
+    if ((u32)(er - 823) > 400u || larger(ee, ev) > 1623 || (u32)(eh - 873) > 300u || (u32)(emu - 923) > 200u)
         return false;
-    // dimensionless parameters as significands x 2^exponent (each product's
-    // error is ~2^-59 of it)
-    int half;
-    const u64 r = rsqrt62(rb, er, half);                                 // 1/r0 = r 2^(-62 - half)
-    const u64 hM = significand62(hb);
+    const bool neg = (eb >> 63) != 0;
+
+    // 1/r0 = r 2^(-62 - half), r = mant^(-1/2) with r0^2 = mant 4^half, mant in
+    // [1, 4): FP32 seed y = My 2^-24, e = 1 - mant y^2 in Q60, y (1 + e/2 + 3 e^2/8)
+    const int odd = (er + 1) & 1, half = (er - 1023 - odd) / 2;
+    const u64 rx = significand62(rb) >> (1 - odd);                       // mant 2^61
+    const float yf = rsqrt_f32(mul(u32_to_f32(hi32(rx)), 1.0f / 536870912.0f));
+    const u32 My = f32_to_u32(mul(yf, 16777216.0f));
+    const i64 ey = (i64)((1ull << 60) - mulhi(rx, ((u64)My * My) << 15));
+    const i32 eyh = (i32)(ey >> 13);                                     // Q47
+    const i64 U = (ey >> 1) + ((3 * (((i64)eyh * eyh) >> 34)) >> 3);     // Q60
+    const u64 r = ((u64)My << 38) + (u64)(((i64)My * U + 0x200000) >> 22);
+
+    // dimensionless parameters, in FP32 for the domain and the start
+    const u64 hM = significand62(hb), muM = significand62(mb);
+    const float s30 = 1.0f / 1073741824.0f;
+    const float hf = mul(u32_to_f32(hi32(hM)), s30), hy = mul(hf, yf), hy2 = mul(hy, hy);
+    const int kw = eh - 1023 - half;
+    const u64 vM = significand62(vb), eM = significand62(eb);
+    const float mf = mul(mul(mul(u32_to_f32(hi32(muM)), s30), mul(yf, hy2)), power2(emu - 1023 + 2 * kw - half));
+    const float Vf = mul(mul(mul(u32_to_f32(hi32(vM)), s30), hy2), power2(larger(ev - 1023 + 2 * kw, -200)));
+    const float am = mul(mul(mul(u32_to_f32(hi32(eM)), s30), mul(hy, yf)), power2(larger(ee - 1023 + kw - half, -200)));
+    const float af = neg ? -am : am, bf = sub(Vf, mf), Bf = fma(2.0f, mf, -Vf);
+    // (comparisons that are false for NaN)
+    if (!(Vf < mul(1.9998f, mf) && Vf < 3.99f && mf < 3.99f && am < 0.999f && bf < 1.999f && bf > -1.999f && Bf < 1.999f))
+        return false;
+
+    // and as significands x 2^exponent (each product's error is ~2^-59 of it)
     const u64 wM = mulhi(hM, r) << 2;                                    // h/r0 = wM 2^(eh - 1085 - half)
     const u64 kM = mulhi(wM, r) << 2;                                    // h/r0^2 = kM 2^(eh - 1085 - 2 half)
     const u64 w2M = mulhi(wM, wM) << 1;                                  // (h/r0)^2 = w2M 2^(2 eh - 2107 - 2 half)
-    const u64 nM = mulhi(significand62(mb), r) << 2;                     // mu/r0 = nM 2^(emu - 1085 - half)
+    const u64 nM = mulhi(muM, r) << 2;                                   // mu/r0 = nM 2^(emu - 1085 - half)
     int ej = emu + eh - 2106 - 3 * half, em = emu + 2 * eh - 3128 - 3 * half;
     int ea = ee + eh - 2106 - 2 * half, eV = ev + 2 * eh - 3128 - 2 * half;
     const u64 jM = normalize(mulhi(nM, kM), ej);                         // mu h/r0^3 = jM 2^(ej)
     const u64 mM = normalize(mulhi(nM, w2M), em);                        // m = mM 2^(em)
-    const u64 aM = normalize(mulhi(significand62(eb), kM), ea);          // |a| = aM 2^(ea)
-    const u64 VM = normalize(mulhi(significand62(vb), w2M), eV);         // V = VM 2^(eV)
+    const u64 aM = normalize(mulhi(eM, kM), ea);                         // |a| = aM 2^(ea)
+    const u64 VM = normalize(mulhi(vM, w2M), eV);                        // V = VM 2^(eV)
 
-    // bound orbit, V < 2 m (1 - 2^-13), compared at the significands' own scales
-    const u32 vh = hi32(VM), mh = hi32(mM), mlim = mh - (mh >> 13);
-    const int dV = eV - em;                                              // V/m = VM/mM 2^dV
-    const u32 vlim = dV == 0 ? 2 * mlim : (dV == 1 ? mlim : 0u);
     // parameters in fixed point: |a| in Q62, m and V in Q61
-    const int sa = -62 - ea, sm = -61 - em, sV = -61 - eV;
-    if (!(dV < 0 || vh < vlim) || sa < 0 || sm < 0 || sV < 0) return false;
-    const u64 amag = aM >> shift63(sa), mq = mM >> shift63(sm), Vq = VM >> shift63(sV);
-
     const u64 one60 = 1ull << 60, one62 = 1ull << 62;
-    const bool neg = (eb >> 63) != 0;
+    const u64 amag = aM >> shift63(-62 - ea), mq = mM >> shift63(-61 - em), Vq = VM >> shift63(-61 - eV);
     const u64 a1 = neg ? one62 - amag : one62 + amag;                    // a + 1, Q62
     const u64 b2 = Vq - mq + one62;                                      // b + 2, Q61
     i64 Bs = (i64)(2 * mq - Vq);                                         // Q61
     Bs = Bs < 0 ? 0 : Bs;
     const u64 B = (u64)Bs << 1;                                          // Q62
-    const float am = mul(u32_to_f32(hi32(amag)), 1.0f / 1073741824.0f), af = neg ? -am : am;
-    const float bf = fma(u32_to_f32(hi32(b2)), 1.0f / 536870912.0f, -2.0f);
-    const float Bf = mul(u32_to_f32(hi32((u64)Bs)), 1.0f / 536870912.0f);
-    if (!(amag < one62 - (one62 >> 10) && bf < 1.999f && bf > -1.999f && Bf < 1.999f)) return false;
     const float sf = start(af, bf, Bf);
     if (!(sf > 0.5625f && sf < 1.75f && mul(Bf, mul(sf, sf)) < 1.99f)) return false;
     const u32 sh = f32_to_u32(mul(sf, 1073741824.0f)) - 724u;                // Q30, 2^-20.5 low

@@ -7,7 +7,7 @@
 // takes one cycle.  A kick changes a velocity by a small part of itself, so
 // its terms do not need the velocity's own 53 bits: a float pair (hi + lo, 48
 // bits, error-free products by FMA) leaves an error of 2^-45 of the kick,
-// below 2^-54 of the velocity for any kick this form accepts (2^-11 of the
+// below 2^-55 of the velocity for any kick this form accepts (2^-10 of the
 // velocity), against the 2^-54 that each of the FP64 form's seven additions
 // to the velocity made.  The kick's terms are summed apart from the velocity
 // and reach it in one FP64 addition.  Measured against 113-bit arithmetic the

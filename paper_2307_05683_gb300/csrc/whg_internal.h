@@ -126,7 +126,25 @@ struct WhgAdj {
 struct WhgLaunch {
     int grid, block;
     cudaStream_t stream;
+    int sms;                         // SMs the launch has (0: all of the device's)
 };
+
+// Warps of bucket b, and of all buckets, with four lanes per planet (whg_wide.cuh).
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+inline int whg_wide_warps_of(const WhgBuckets& bk, int b)
+{
+    const int per = 32 / bk.L[b] / 4;                    // systems per warp
+    return (bk.sys0[b + 1] - bk.sys0[b] + per - 1) / per;
+}
+
+inline int whg_wide_warps(const WhgBuckets& bk)
+{
+    int n = 0;
+    for (int b = 0; b < bk.nb; ++b) n += whg_wide_warps_of(bk, b);
+    return n;
+}
 
 // Kernel launchers (whg_kernels_common.cu, whg_kernels_nt6.cu, whg_kernels_nt8.cu).
 cudaError_t whg_launch_init(const WhgState&, const WhgBuckets&, const WhgIn&, const WhgLaunch&);
@@ -151,6 +169,8 @@ cudaError_t whg_launch_step_nt6(const WhgState&, const WhgBuckets&, long long, i
 cudaError_t whg_launch_step_nt8(const WhgState&, const WhgBuckets&, long long, int, const WhgLaunch&);
 cudaError_t whg_launch_step_few_nt6(const WhgState&, const WhgBuckets&, long long, int, const WhgLaunch&);
 cudaError_t whg_launch_step_few_nt8(const WhgState&, const WhgBuckets&, long long, int, const WhgLaunch&);
+cudaError_t whg_launch_step_wide_nt6(const WhgState&, const WhgBuckets&, long long, int, const WhgLaunch&);
+cudaError_t whg_launch_step_wide_nt8(const WhgState&, const WhgBuckets&, long long, int, const WhgLaunch&);
 cudaError_t whg_launch_step_queue_nt6(const WhgState&, const WhgBuckets&, long long, int, const WhgQueue&,
                                       cudaStream_t);
 cudaError_t whg_launch_step_queue_nt8(const WhgState&, const WhgBuckets&, long long, int, const WhgQueue&,

@@ -154,26 +154,47 @@ cudaError_t whg_launch_raw(const WhgState& st, const WhgBuckets& bk, const WhgOu
     return cudaGetLastError();
 }
 
-// Up to 8 warps per SM (2 per sub-partition) a step is bound by each warp's own
-// chain of instructions, and the kernel with more registers is the faster one;
-// above, the resident warps count.  Measured, 8-planet systems, us per step, few /
-// many: 2432 systems (4 warps per SM) 4.21 / 4.76, 4096 (6.7) 4.82 / 5.33,
-// 8192 (13.5) 9.1 / 7.98.  Results are the same bits.
-bool whg_few_warps(const WhgBuckets& bk)
+static int sm_count()
 {
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
         cudaGetLastError();
-        return false;
+        return 0;
     }
-    return bk.warp0[bk.nb] <= 8 * sms;
+    return sms;
 }
+
+// Three step kernels, the same bits from each (whg_wide.cuh, step_body):
+// * four lanes per planet while its warps, four times as many, stay within 8
+//   per SM (2 per sub-partition), or 12 for systems of 6 or more planets, whose
+//   pair rounds it saves most.  us per step, four lanes / one: 8 planets 608
+//   systems (4 warps per SM) 2.22 / 4.21, 1216 (8) 2.82 / 4.21, 1824 (12)
+//   3.61 / 4.19, 2432 (16) 5.54 / 4.19; 5 planets 777 (5) 2.89 / 3.60,
+//   1500 (10) 3.61 / 3.60; 2 planets 4864 (8) 2.49 / 2.89, 9728 (16) 5.25 / 2.94;
+// * one lane per planet, registers for one warp's own chain of instructions
+//   (178; k_step<.., 1>), up to 8 warps per SM;
+// * one lane per planet, 128 registers, above: the resident warps count.  178 /
+//   128 registers: 2432 systems (4 warps per SM) 4.21 / 4.76, 4096 (6.7) 4.82 /
+//   5.33, 8192 (13.5) 9.1 / 7.98.
+static bool wide_warps(const WhgState& st, const WhgBuckets& bk, int sms)
+{
+    if (st.full_rotation) return false;              // interaction schedule without reactions: FP64 only
+    int least = 8;
+    for (int b = 0; b < bk.nb; ++b) least = bk.L[b] < least ? bk.L[b] : least;
+    return whg_wide_warps(bk) <= (least >= 6 ? 12 : 8) * sms;
+}
+
+bool whg_few_warps(const WhgBuckets& bk) { return bk.warp0[bk.nb] <= 8 * sm_count(); }
 
 cudaError_t whg_launch_step(const WhgState& st, const WhgBuckets& bk, long long n, int newton_terms,
                             int gr_mode, const WhgLaunch& l)
 {
-    if (whg_few_warps(bk))
+    const int sms = l.sms > 0 ? l.sms : sm_count();
+    if (wide_warps(st, bk, sms))
+        return newton_terms == 6 ? whg_launch_step_wide_nt6(st, bk, n, gr_mode, l)
+                                 : whg_launch_step_wide_nt8(st, bk, n, gr_mode, l);
+    if (bk.warp0[bk.nb] <= 8 * sms)
         return newton_terms == 6 ? whg_launch_step_few_nt6(st, bk, n, gr_mode, l)
                                  : whg_launch_step_few_nt8(st, bk, n, gr_mode, l);
     return newton_terms == 6 ? whg_launch_step_nt6(st, bk, n, gr_mode, l)

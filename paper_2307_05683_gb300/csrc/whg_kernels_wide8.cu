@@ -1,0 +1,16 @@
+// whg_kernels_wide8.cu -- the step kernel for small ensembles, 8-term Stumpff series.
+#include "whg_wide.cuh"
+
+cudaError_t whg_launch_step_wide_nt8(const WhgState& st, const WhgBuckets& bk, long long n, int gr_mode,
+                                     const WhgLaunch& l)
+{
+    const long long threads = (long long)whg_wide_warps(bk) * 32;
+    const int grid = (int)((threads + l.block - 1) / l.block);
+    if (gr_mode == 0)
+        whg::k_step_wide<8, 0><<<grid, l.block, 0, l.stream>>>(st, bk, n);
+    else if (gr_mode == 1)
+        whg::k_step_wide<8, 1><<<grid, l.block, 0, l.stream>>>(st, bk, n);
+    else
+        whg::k_step_wide<8, 2><<<grid, l.block, 0, l.stream>>>(st, bk, n);
+    return cudaGetLastError();
+}

@@ -146,6 +146,7 @@ extern "C" int whg_integrate_noalloc(int n_systems, int max_planets, const whg_o
     l.block = block;
     l.grid = (int)((NL + block - 1) / block);
     l.stream = (cudaStream_t)cuda_stream;
+    l.sms = 0;
 
     // The init kernel writes every lane and per-system field read later
     // (status and step counters start at zero), so stale contents left by an
