@@ -245,7 +245,9 @@ int whg_adjoint_backward(whg_ctx* ctx, const double* loss_weight, double* grad_p
  * whg_adjoint_forward.
  * sm_split: -1 (default): split the SMs into two green contexts when the
  *   ensemble's warps need at most half of the SMs at one warp per SM
- *   sub-partition (about 1200 8-planet systems or fewer on a 152-SM GPU).
+ *   sub-partition, and more than a third of all sub-partitions (about 800 to
+ *   1200 8-planet systems on a 152-SM GPU; smaller ensembles leave room for
+ *   every kernel without it).
  *   In the backward half the back kernels, its critical path, then run on
  *   ceil(warps / 4) SMs (rounded up to the partition granularity, 8 SMs on
  *   this GPU), one warp per sub-partition, and the tape kernels on the

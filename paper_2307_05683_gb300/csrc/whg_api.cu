@@ -985,18 +985,21 @@ static int leave_stream(whg_ctx* c, cudaStream_t s, CUcontext x)
     return WHG_OK;
 }
 
-// SMs wanted for the chain partition (0: no split) for this ensemble.
-static int chain_sms_wanted(const whg_ctx* c)
+// Whether one back kernel and two tape kernels leave every SM sub-partition at
+// most one warp.  They then hardly ever meet on one, split or not.
+static bool roomy(const whg_ctx* c, int sms) { return 3 * c->bk.warp0[c->bk.nb] <= 4 * sms; }
+
+// SMs wanted for the chain partition (0: no split) for this ensemble.  Making
+// and releasing the partition costs a context about 1.4 ms, so a roomy
+// ensemble does without: a whole gradient call on a new context, 8 systems x 50
+// steps 2.5 -> 1.1 ms, 200 x 200 5.1 -> 3.5 ms, and on a kept one 200 x 200
+// 3.17 -> 3.09 ms.
+static int chain_sms_wanted(const whg_ctx* c, int sms)
 {
     if (c->cfg_split == 0) return 0;
-    int sms = 0;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess) {
-        cudaGetLastError();
-        return 0;
-    }
     const int warps = c->bk.warp0[c->bk.nb];
     const int want = c->cfg_split > 0 ? c->cfg_split : (warps + 3) / 4;   // one warp per sub-partition
-    if (c->cfg_split < 0 && 2 * want > sms) return 0;                      // the forward fills the GPU
+    if (c->cfg_split < 0 && (2 * want > sms || roomy(c, sms))) return 0;   // the forward fills the GPU, or room for all
     if (want >= sms) return 0;
     return want;
 }
@@ -1044,8 +1047,11 @@ int whg_adjoint_forward(whg_ctx* c, long long n_steps, int checkpoint_every, con
     const size_t tape_bytes = tape_len * sizeof(double);
     // the partition, then the tape pool: with the split and a tape budget, a
     // buffer per segment where they fit (half of the free memory, or the cap)
-    const int want = chain_sms_wanted(c);
+    int sms = 0;
+    WHG_CUDA(c, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device));
+    const int want = chain_sms_wanted(c, sms);
     c->split = want > 0 && make_split(c, want);
+    const bool beside = c->split || roomy(c, sms);         // tapes beside the forward half's last segments
     const bool pre = c->split && c->cfg_tape_bytes != 0;   // tapes beside the forward half
     long long nbuf = WHG_TAPE_BUFFERS;
     if (pre) {
@@ -1092,26 +1098,32 @@ int whg_adjoint_forward(whg_ctx* c, long long n_steps, int checkpoint_every, con
     c->adj_ready = false;
     WHG_CUDA(c, cudaMemcpyAsync(tcopy, target, tgt * sizeof(double), cudaMemcpyDeviceToDevice, c->stream));
     // Segments whose tapes are recomputed beside the forward half: with a tape
-    // budget all that have a buffer, else (split) the last nbuf - 1, which the
-    // first back kernels need at once.  From segment `from` on, the forward
-    // runs on the first partition, so that no tape kernel shares its SMs.
-    const long long npre = !c->split ? 0 : pre ? (nbuf < nseg ? nbuf : nseg)
-                                                : (nbuf - 1 < nseg ? nbuf - 1 : nseg);
+    // budget all that have a buffer, else (split, or room for all kernels) the
+    // last nbuf - 1, which the first back kernels need at once.  From segment
+    // `from` on, a split forward runs on the first partition, so that no tape
+    // kernel shares its SMs.
+    const long long npre = !beside ? 0 : pre ? (nbuf < nseg ? nbuf : nseg)
+                                              : (nbuf - 1 < nseg ? nbuf - 1 : nseg);
     const long long first_pre = nseg - npre, from = pre ? 0 : first_pre;
     const CUcontext xt = c->split ? c->x_tape : nullptr;
+    const cudaStream_t ts[2] = {tape_cfg(c, 0).stream, tape_cfg(c, 1).stream};
     WhgLaunch l = chain_cfg(c, false);
     CUcontext xc = nullptr;
     bool switched = false;
     for (long long seg = 0; seg <= nseg; ++seg) {
-        if (c->split && seg == from) {                  // onto the partition
+        if (beside && seg == from) {
             WHG_CUDA(c, cudaEventRecord(c->ev_entry, c->stream));
-            for (cudaStream_t s : {c->s_chain, c->s_tape[0], c->s_tape[1]}) {
-                rc = enter_stream(c, s, s == c->s_chain ? c->x_chain : xt);
+            for (int i = 0; i < 2; ++i) {
+                rc = enter_stream(c, ts[i], xt);
                 if (rc) return rc;
             }
-            l = chain_cfg(c, true);
-            xc = c->x_chain;
-            switched = true;
+            if (c->split) {                              // onto the partition
+                rc = enter_stream(c, c->s_chain, c->x_chain);
+                if (rc) return rc;
+                l = chain_cfg(c, true);
+                xc = c->x_chain;
+                switched = true;
+            }
         }
         {
             WHG_SCOPE(xc, save);
@@ -1123,7 +1135,7 @@ int whg_adjoint_forward(whg_ctx* c, long long n_steps, int checkpoint_every, con
         if (seg >= first_pre) {
             WHG_SCOPE(xt, tape);
             const int i = (int)(seg % 2);
-            WHG_CUDA(c, cudaStreamWaitEvent(c->s_tape[i], c->ev_ckpt, 0));
+            WHG_CUDA(c, cudaStreamWaitEvent(ts[i], c->ev_ckpt, 0));
             rc = launch_tape(c, a, (int)seg, i);
             if (rc) return rc;
         }
@@ -1140,8 +1152,12 @@ int whg_adjoint_forward(whg_ctx* c, long long n_steps, int checkpoint_every, con
         if (rc) return rc;
     }
     if (switched) {
-        for (cudaStream_t s : {c->s_chain, c->s_tape[0], c->s_tape[1]}) {
-            rc = leave_stream(c, s, s == c->s_chain ? c->x_chain : xt);
+        rc = leave_stream(c, c->s_chain, c->x_chain);
+        if (rc) return rc;
+    }
+    if (beside) {
+        for (int i = 0; i < 2; ++i) {
+            rc = leave_stream(c, ts[i], xt);
             if (rc) return rc;
         }
     }
