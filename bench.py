@@ -54,6 +54,12 @@ START_FLOPS = {(8, 8, 1): 776, (8, 8, 0): 776, (8, 6, 1): 776, (8, 8, 2): 776}
 ALG_FLOPS_BY_PLANETS = {1: 349, 2: 722, 3: 1119, 4: 1540, 5: 1985, 6: 2454, 7: 2947, 8: 3464}
 
 
+# Flops of one system-step that run on the FP64 pipe, FMA = 2 (ncu on the bench
+# launch: 208 FMA, 72 additions, 40 products); the rest of the algorithm runs on
+# the integer and FP32 pipes.
+FP64_PIPE_FLOPS = 528
+
+
 def fp64_flops(gr_mode: int, halley_fp32: bool, newton_terms: int = 8) -> int:
     key = (8, newton_terms, gr_mode)
     return ALG_FLOPS[key] - (START_FLOPS[key] if halley_fp32 else 0)
@@ -76,8 +82,7 @@ def parse_args():
     p.add_argument("--chunk", type=int, default=10000, help="integrator steps per benchmark step")
     p.add_argument("--gr-mode", type=int, default=1)
     p.add_argument("--halley-fp32", type=int, choices=[0, 1], default=0,
-                   help="Kepler solver's initial guess and Halley steps in FP32 (1, an option) "
-                        "or FP64 (0, the library default: every step in FP64)")
+                   help="passed to the library, where it has no effect any more")
     p.add_argument("--block-size", type=int, default=0)
     p.add_argument("--e2e-steps", type=int, default=5)
     p.add_argument("--cpu-seconds", type=float, default=15.0, help="CPU work of the oracle sample")
@@ -95,12 +100,9 @@ def workload(args) -> dict:
             "systems_per_gpu": args.systems, "planets": 8,
             "integrator_steps_per_bench_step": args.chunk,
             "gr_mode": args.gr_mode, "newton_terms": 8, "halley_terms": 4,
-            "kepler_solver": ("initial guess + 2 Halley steps (4-term series) in FP32, 2 Newton steps "
-                              "(8-term series) and f, g in FP64" if args.halley_fp32 else
-                              "initial guess, 2 Halley steps (4-term series), 2 Newton steps (8-term series) "
-                              "and f, g all in FP64"),
-            "l2": "state register-resident during each 100-step work unit (reloaded from L2 between units); "
-                  "256 MB L2 flush between timed steps"}
+            "kepler_solver": "start (2 Halley steps, 4-term series) in FP32, one third-order step with 8-term "
+                             "series and f, g in 64-bit fixed point; vectors in FP64",
+            "l2": "state register-resident during each launch; 256 MB L2 flush between timed steps"}
 
 
 # ------------------------------------------------------------ environment --
@@ -347,7 +349,7 @@ def measure_uneven(whg, torch, systems=1 << 16, steps=20000, seed=303):
     Rates count every system for every
     step (a frozen system counts but costs nothing once its whole warp is
     frozen); CUDA events on the library's stream after a warm-up of 1600
-    steps.  The FP64 fraction counts the algorithmic flops of each system's
+    steps.  The algorithmic rate counts the flops of each system's
     planet count (idle lanes do none), every system every step."""
     ens = inputs.compact_ensemble(seed, systems)
     stream = torch.cuda.Stream()
@@ -372,7 +374,7 @@ def measure_uneven(whg, torch, systems=1 << 16, steps=20000, seed=303):
         it.close()
         rate = systems * steps / (ms / 1e3)
         out[name] = {"system_steps_per_s": round(rate, 1), "stopped": int((st != 0).sum()),
-                     "frac": round(rate * flops / 1e12 / FP64_PEAK_TFLOPS, 4)}
+                     "algorithmic_tflops": round(rate * flops / 1e12, 4)}
     return out
 
 
@@ -397,22 +399,19 @@ def throughput_sweep(whg, torch, sizes=tuple(1 << k for k in range(14, 21)), win
         cfg = {k: best[k] for k in ("block_size", "queue_steps", "steps_per_launch", "graph_launches")}
         rate, n = time_rate(whg, torch, ens, window_s, stream, min_steps=min_steps, gr_mode=1, **cfg)
         out.append({"systems": S, "steps": n, "system_steps_per_s": round(rate, 1),
-                    "frac": round(rate * fp64_flops(1, False) / 1e12 / FP64_PEAK_TFLOPS, 4),
+                    "algorithmic_tflops": round(rate * fp64_flops(1, False) / 1e12, 4),
                     "config": cfg, "candidates_timed": best["tried"]})
     return out
 
 
 def solver_comparison(whg, torch, ens, gr_mode: int, window_s=1.0):
-    """The bench workload with the whole Kepler solver in FP64 (the paper's
-    arithmetic) beside the default FP32 starting phase, same timing method."""
+    """The bench workload with and without the halley_fp32 option (which has no
+    effect any more), same timing method."""
     stream = torch.cuda.Stream()
     out = {}
     for h32 in (False, True):
         rate, n = time_rate(whg, torch, ens, window_s, stream, gr_mode=gr_mode, halley_fp32=h32)
-        fl = fp64_flops(gr_mode, h32)
-        out["fp32_start" if h32 else "all_fp64"] = {
-            "system_steps_per_s": round(rate, 1), "steps": n, "fp64_flops_per_system_step": fl,
-            "frac": round(rate * fl / 1e12 / FP64_PEAK_TFLOPS, 4)}
+        out["halley_fp32" if h32 else "default"] = {"system_steps_per_s": round(rate, 1), "steps": n}
     return out
 
 
@@ -505,9 +504,10 @@ def run_whg(args):
             dist.destroy_process_group()
         return
 
-    flops = fp64_flops(args.gr_mode, bool(args.halley_fp32))
+    flops = fp64_flops(args.gr_mode, False)
     kernel_ms = total_ms / args.steps / max(launches_per_step, 1.0)
-    achieved = flops * S * (chunk / max(launches_per_step, 1.0)) / (kernel_ms / 1e3) / 1e12
+    kernel_rate = S * (chunk / max(launches_per_step, 1.0)) / (kernel_ms / 1e3)
+    achieved = FP64_PIPE_FLOPS * kernel_rate / 1e12
     adjoint = measure_adjoint(whg, torch) if world == 1 else None
     sweep = throughput_sweep(whg, torch) if world == 1 else None
     solvers = solver_comparison(whg, torch, ens, args.gr_mode) if world == 1 else None
@@ -515,9 +515,10 @@ def run_whg(args):
     roofline = {"bound": "alu", "achieved": round(achieved, 4), "peak": round(FP64_PEAK_TFLOPS, 4),
                 "unit": "TFLOP/s", "frac": round(achieved / FP64_PEAK_TFLOPS, 4),
                 "traffic": profiled_traffic(),
-                "kernel": "k_step_queue<8,1> via queue_unit (FP64 pipe)",
+                "kernel": "k_step<8,1,1>",
+                "fp64_pipe_flops_per_system_step": FP64_PIPE_FLOPS,
                 "algorithmic_flops_per_system_step": flops,
-                "fp32_flops_per_system_step": START_FLOPS[(8, 8, args.gr_mode)] if args.halley_fp32 else 0,
+                "algorithmic_tflops": round(flops * kernel_rate / 1e12, 4),
                 "peak_basis": "recipe unit counts x clocks: 152 SMs x 2 FP64 FMA/clk x 2 x 2.07 GHz"}
     line = {"metric": METRIC, "value": round(value, 1), "unit": UNIT, "n_gpus": world,
             "steps": args.steps, "warmup": args.warmup, "ms_per_step": round(total_ms / args.steps, 4),
