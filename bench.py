@@ -150,7 +150,7 @@ def kernel_source_hash() -> str:
     instantiation with 8-term Newton-phase series), comments excluded."""
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_2307_05683_gb300", "csrc")
-    for name in ("whg_device.cuh", "whg_kernels_nt8.cu"):
+    for name in ("whg_device.cuh", "whg_fixed.cuh", "whg_interact.cuh", "whg_kernels_few8.cu"):
         h.update(name.encode())
         h.update(code_only(open(os.path.join(csrc, name)).read()).encode())
     return h.hexdigest()[:16]

@@ -3,25 +3,28 @@
 // warp lanes per system (one lane per planet, L in 1..8, floor(32/L) systems
 // per warp).
 //
-// Why the code looks as it does.  The whole step is FP64 arithmetic on a few registers
-// per lane; on this part the FP64 pipe retires about 2 lanes per clock per SM
-// while FP32, integer, shuffle and MUFU work retire tens of times faster.  So
-// the step is bound by the number of FP64 instructions alone, and the code
-// spends integer and FP32 work freely to save FP64 instructions:
+// Why the code looks as it does.  An FP64 warp instruction holds its pipe for
+// 64 cycles (76 with all four sub-partitions busy), an FP32 one its pipe for 1, an
+// integer one for 2 to 6.  So a step spends FP64 only on what needs a double's
+// rounding, 40 instructions per planet, and the rest elsewhere at no less
+// precision:
+//   * Kepler's equation is solved in 64-bit fixed point (whg_fixed.cuh) and the
+//     interaction's terms are float pairs (whg_interact.cuh), each with an FP64
+//     form out of line for the states it does not hold;
 //   * reciprocals and reciprocal square roots start from the FP32 hardware
 //     approximation of a mantissa built with integer operations and take one
 //     third-order refinement whose correction (from the exact 1 - x y or
 //     1 - x y^2) is formed in fixed point on the integer pipe, leaving one
-//     FP64 FMA per call, and the solver's factors -1/2 are exponent
-//     decrements;
+//     FP64 FMA per call;
 //   * the all-pairs interaction uses Newton's third law (Sec. 3.3), with
 //     partner schedules that suit warp shuffles rather than AVX512 lanes;
 //   * cross-lane sums of 3-vectors are reduce-scatters by xor partners when L
 //     is 4 or 8 (Sec. 3.4 reduces with a butterfly), else gathers in fixed
 //     lane order; either way every lane gets the bitwise-identical total;
-//   * a persistent work queue moves (warp-group, steps) units between SMs so
-//     that no SM finishes late.
-// State stays in registers during a unit of steps; HBM is touched only at
+//   * small ensembles take four lanes per planet (whg_wide.cuh), large ones a
+//     kernel with fewer registers, or a persistent work queue that moves
+//     (warp-group, steps) units between SMs.
+// State stays in registers during a launch; HBM is touched only at
 // load and store (coalesced: consecutive lanes read consecutive doubles).
 #pragma once
 
@@ -66,10 +69,8 @@ __device__ __forceinline__ float approx_rsqrt_f32(float x)
 }
 
 // ------------------------------------------------------------------------
-// Integer-pipe pieces of the reciprocal and reciprocal square root.  On this
-// GPU an FP64 warp instruction holds the FP64 pipe for 64 cycles and an
-// integer one its pipe for about 1, so integer forms replace FP64 operations
-// wherever the operands are short: the seeds y below carry 24 significant
+// Integer-pipe pieces of the reciprocal and reciprocal square root: integer
+// forms replace FP64 operations wherever the operands are short: the seeds y below carry 24 significant
 // bits (an FP32 approximation widened to FP64).
 
 // D 2^-s rounded to the nearest double (ties to even); D a signed 64-bit
