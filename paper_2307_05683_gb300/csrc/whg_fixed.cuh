@@ -186,8 +186,11 @@ WHG_HD i64 to_fixed(u64 bits, int sh)
 
 WHG_HD int larger(int a, int b) { return a > b ? a : b; }
 
-// 2^k as a float, 0 below 2^-126 (k < 128).
-WHG_HD float power2(int k) { return bits_to_f32(k < -126 ? 0u : (u32)(k + 127) << 23); }
+WHG_HD int smaller(int a, int b) { return a < b ? a : b; }
+
+// 2^k as a float, 0 below 2^-126 and infinity from 2^128 on (solve's exponent
+// guards let k reach about +-1000: a speed of 2^300, a step of 2^150).
+WHG_HD float power2(int k) { return bits_to_f32(k < -126 ? 0u : (u32)(smaller(k, 128) + 127) << 23); }
 
 // Series coefficients 4^k/n! as round(4^k 2^q / n!), from an exact division.
 constexpr u64 coef(int k, int n, int q)
@@ -387,7 +390,7 @@ WHG_HD bool solve(double mu, double h, double r0sq, double eta0, double v2, Solu
     if (!(d1 < (1ll << 40) && d1 > -(1ll << 40))) return false;
     const i64 e1 = d1 >> 13;                                             // Q47
     const i64 t = d1 + (((i64)(i32)e1 * (i32)e1) >> 34);                    // Q60
-    const u64 yn = y + mulhi((u64)((t << 4) + (1ll << 48)), y) - (y >> 16);                  // Q62
+    const u64 yn = y + mulhi(((u64)t << 4) + (1ull << 48), y) - (y >> 16);                  // Q62
 
     const u64 mg3 = mulhi(mq, G3 << 2);                                  // Q60
     if (mg3 >= one60 - (one60 >> 6)) return false;
