@@ -23,3 +23,31 @@ def test_unresolved_steps_of_any_size_are_left_out(lib, log2r, log2h, log2mu):  
     r, h, mu = 2.0 ** log2r, 2.0 ** log2h, 2.0 ** log2mu
     for v2 in (0.0, 0.25 * mu / r, mu / r):
         assert not lib.fixed_solve(8, mu, h, r * r, 0.0, v2, out.ctypes.data)
+
+
+@pytest.mark.parametrize("T", [6, 8])
+@pytest.mark.parametrize("zmin", [0.0, 0.5, 1.0, 1.5])
+def test_coefficients_over_the_whole_domain(lib, T, zmin):  # noqa: F811
+    """m, V and a drawn over all that the solver takes (z from zmin to zmin +
+    0.5).  1 - f, fdot and 1 - gdot are one rounding (2^-53 of the value at
+    most, 0.43 2^-53 rms and no mean) away from a value of 55 correct bits, and
+    unbiased: mean within 2^-57 and the sample's own scatter.  g is h times a
+    difference from 1 of such a value, so it is judged against h."""
+    rng = np.random.default_rng(21)
+    out, err, kept = np.zeros(9), np.zeros(9), []
+    while len(kept) < 3000:
+        m = rng.uniform(0, 4)
+        V, a = 2 * m * rng.uniform(), rng.uniform(-1, 1)
+        r0 = rng.uniform(1, 2)
+        h = np.sqrt(m * r0 ** 3)
+        x = (1.0, h, r0 * r0, a * r0 * r0 / h, V * r0 * r0 / (h * h))
+        if a * a > V or not lib.fixed_solve(T, *x, out.ctypes.data):
+            continue
+        z = (2 * m - V) * out[4] ** 2
+        if zmin <= z < zmin + 0.5:
+            lib.errors(T, *x, out.ctypes.data, err.ctypes.data)
+            kept.append([err[0], err[1] * out[1] / h, err[2], err[3]])
+    e = np.asarray(kept) * 2.0 ** 53
+    assert np.abs(e).max() <= 1.25, np.abs(e).max(axis=0)
+    assert np.sqrt((e ** 2).mean(axis=0)).max() <= 0.5
+    assert np.all(np.abs(e.mean(axis=0)) <= 2.0 ** -4 + 4 * e.std(axis=0) / np.sqrt(len(e))), e.mean(axis=0)
