@@ -588,7 +588,8 @@ __device__ __forceinline__ MassSum mass_sum(const Group<L>& g, double m, double 
         s.k = k;
         gather3<L>(g, k, s.x, s.y, s.z);
     } else {
-        group_sum3<L>(g, m * x, m * y, m * z, s.x, s.y, s.z);
+        // (products that the additions never absorb: every kernel sums the same bits)
+        group_sum3<L>(g, __dmul_rn(m, x), __dmul_rn(m, y), __dmul_rn(m, z), s.x, s.y, s.z);
     }
     return s;
 }
@@ -690,9 +691,9 @@ __device__ __forceinline__ bool kick(const Group<L>& g, double qx, double qy, do
             vy = fma(c, qy, vy);
             vz = fma(c, qz, vz);
         } else {
-            const double ax = c * qx, ay = c * qy, az = c * qz;
+            const double ax = __dmul_rn(c, qx), ay = __dmul_rn(c, qy), az = __dmul_rn(c, qz);
             double bx, by, bz;
-            group_sum3<L>(g, mrat * ax, mrat * ay, mrat * az, bx, by, bz);
+            group_sum3<L>(g, __dmul_rn(mrat, ax), __dmul_rn(mrat, ay), __dmul_rn(mrat, az), bx, by, bz);
             vx = vx + (ax - bx);
             vy = vy + (ay - by);
             vz = vz + (az - bz);

@@ -156,12 +156,19 @@ WHG_HD void accumulate(Pair& s, float h, float l)
     s.l = add(s.l, add(t.l, l));
 }
 
-// The double hi 24 + lo bits (truncated float and the rest) of a constant.
+// a - b, never contracted with the product that a may be.
+#if defined(__CUDA_ARCH__)
+__device__ __forceinline__ double sub64(double a, double b) { return __dsub_rn(a, b); }
+#else
+inline double sub64(double a, double b) { volatile double r = a - b; return r; }
+#endif
+
+// A constant as a float and the rest of it (24 + 24 bits).
 WHG_HD Pair split(double x)
 {
     Pair r;
     r.h = (float)x;
-    r.l = (float)(x - (double)r.h);
+    r.l = (float)sub64(x, (double)r.h);
     return r;
 }
 

@@ -74,7 +74,7 @@ __device__ __forceinline__ double wide_mass_sum(const WideGroup<L>& g, double m,
         if (L == 8) k += __shfl_xor_sync(WHG_FULL_MASK, k, 1);
         return k;
     }
-    return group_sum<L>(g, m * x);
+    return group_sum<L>(g, __dmul_rn(m, x));
 }
 
 // sum_floats of this lane's coordinate.
