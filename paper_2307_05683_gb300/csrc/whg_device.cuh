@@ -711,6 +711,8 @@ struct Masses {
     double m, hm, mrat, jc, kgr;         // mass, dt m, m/m0, jump coefficient, GR coefficient
     pairs::Pair hmp, kgp;                // hm and kgr as float pairs
     pairs::Pair hmj[L > 1 ? L / 2 : 1];  // hm of the partners at distance 1..L/2
+    pairs::Pair mrp;                     // mrat (GR back-reaction)
+    int jm;                              // exponent of jc m and the margin of gr_scale
     unsigned pairs_on;                   // bit k: the partner at distance k holds a planet, and so does this lane
     bool real, full, merged;             // real: this lane holds a planet
 };
@@ -727,6 +729,13 @@ __device__ __forceinline__ Masses<L> masses_of(const Group<L>& g, bool real, dou
     k.kgr = GRM ? (-6.0 * mu * mu * dt) / (c_light * c_light) : 0.0;
     k.hmp = pairs::split(k.hm);
     k.kgp = pairs::split(k.kgr);
+    k.mrp = pairs::split(k.mrat);
+    // a mass that FP32 does not hold: none where it does not count (m < 2^-60 m0),
+    // else GR in FP64 (accept refuses)
+    const int em = fixed::exponent_of(fixed::bits_of(m));
+    const bool holds = em > 923 && em < 1123;
+    k.jm = fixed::exponent_of(fixed::bits_of(k.jc)) + (holds ? em : 900) - 1023 + 24;
+    if (!holds && em + 60 > fixed::exponent_of(fixed::bits_of(mu))) k.kgp.h = __int_as_float(0x7f800000);
     k.real = real;
     k.full = full;
     k.merged = merged;
@@ -767,7 +776,8 @@ __device__ __noinline__ void interact_general(SubStep* r)
 }
 
 // Float sums of (x, y, z) over the system's lanes: this lane's component
-// (L = 4, 8: returned in x) or all three in every lane.
+// (L = 4, 8: returned in x) or all three in every lane.  sum_pairs: the same
+// in float pairs.
 template <int L>
 __device__ __forceinline__ void sum_floats(const Group<L>& g, float& x, float& y, float& z)
 {
@@ -794,6 +804,43 @@ __device__ __forceinline__ void sum_floats(const Group<L>& g, float& x, float& y
     }
 }
 
+template <int L>
+__device__ __forceinline__ pairs::Pair shfl_pair(const pairs::Pair& a, int from)
+{
+    return pairs::Pair{__shfl_sync(WHG_FULL_MASK, a.h, from), __shfl_sync(WHG_FULL_MASK, a.l, from)};
+}
+
+template <int L>
+__device__ __forceinline__ pairs::Pair add_xor(const pairs::Pair& a, const pairs::Pair& send, int o)
+{
+    return pairs::sum(a, pairs::Pair{__shfl_xor_sync(WHG_FULL_MASK, send.h, o), __shfl_xor_sync(WHG_FULL_MASK, send.l, o)});
+}
+
+template <int L>
+__device__ __forceinline__ void sum_pairs(const Group<L>& g, pairs::Pair& x, pairs::Pair& y, pairs::Pair& z)
+{
+    if (L == 4 || L == 8) {
+        constexpr int H = L / 2, Q = L / 4;
+        const pairs::Pair zero = {0.0f, 0.0f};
+        const bool hi = (g.p & H) != 0, mid = (g.p & Q) != 0;
+        const pairs::Pair k0 = add_xor<L>(hi ? z : x, hi ? x : z, H);
+        const pairs::Pair k1 = add_xor<L>(hi ? zero : y, hi ? y : zero, H);
+        pairs::Pair k = add_xor<L>(mid ? k1 : k0, mid ? k0 : k1, Q);
+        if (L == 8) k = add_xor<L>(k, k, 1);
+        x = k;
+    } else if (L > 1) {
+        pairs::Pair s[3] = {{0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}};   // in lane order, the same bits in every lane
+#pragma unroll
+        for (int j = 0; j < L; ++j) {
+            const int from = g.in_group ? g.base + j : g.lane;
+            s[0] = pairs::sum(s[0], shfl_pair<L>(x, from));
+            s[1] = pairs::sum(s[1], shfl_pair<L>(y, from));
+            s[2] = pairs::sum(s[2], shfl_pair<L>(z, from));
+        }
+        x = s[0]; y = s[1]; z = s[2];
+    }
+}
+
 // The largest non-negative x of the system's lanes.
 template <int L>
 __device__ __forceinline__ int group_max(const Group<L>& g, int x)
@@ -809,14 +856,28 @@ __device__ __forceinline__ int group_max(const Group<L>& g, int x)
     return r;
 }
 
+// The velocity scale against which a planet's GR kick is accepted: its own (vl),
+// and no more than leaves the second jump's sum m f, taken in floats, exact
+// enough: an error of about 2^-24 m |f|, of which jc m 2^-24 |f| reaches the
+// positions, below 2^-56 of the planet's own position (e: its exponent; kicks in
+// units of 2^K2).  A position further in is safe too: f falls with r^-3 and the
+// inner planet's own kick is at most 2^-10 of its velocity, which leaves
+// 2^-51 (m/m0)^(1/4) of it at the worst distance.  From exponents alone: jc m is
+// up to 4 times what they say.  (A k far below the exponent range belongs to a
+// planet so close to the star that accept refuses it whatever the scale.)
+__device__ __forceinline__ float gr_scale(float vl, int e, int jm, int K2)
+{
+    return fminf(vl, fixed::bits_to_f32((unsigned)(min(e - jm - K2, 127) + 127) << 23));
+}
+
 // The sub-step with the kick's terms in float pairs (whg_interact.cuh).  Pair
 // rounds as in kick(): distances k < L/2 evaluated by the lower lane of the
 // rotation with the reaction passed back, distance L/2 by both lanes.  The
 // second jump uses that pair kicks leave sum m v unchanged (Newton's third
-// law): its sum is the first one's plus that of the GR kick, which is ~1e-8
-// of it and taken in floats (an error of 1e-15 of the jump's 1e-3 of the
-// position).  Returns false where the form does not hold (for a real lane);
-// the state is then unspecified.
+// law): its sum is the first one's plus that of the GR kick, taken in floats
+// where their 24 bits are enough (gr_scale: the Solar System is 2^20 inside,
+// a Jupiter at 0.05 AU just).  Returns false where the form does not hold (for
+// a real lane); the state is then unspecified.
 template <int L, int GRM, bool Q2>
 __device__ __forceinline__ bool interact_pairs(const Group<L>& g, const Masses<L>& c, double& qx, double& qy, double& qz,
                                                double& vx, double& vy, double& vz, const double* thr2, bool hill,
@@ -837,7 +898,7 @@ __device__ __forceinline__ bool interact_pairs(const Group<L>& g, const Masses<L
         const int ex = fixed::exponent_of(bx), ey = fixed::exponent_of(by), ez = fixed::exponent_of(bz);
         const int ev = max(fixed::exponent_of(fixed::bits_of(vx)),
                            max(fixed::exponent_of(fixed::bits_of(vy)), fixed::exponent_of(fixed::bits_of(vz))));
-        const int eq = group_max<L>(g, c.real ? max(ex, max(ey, ez)) : 0);
+        const int e = max(ex, max(ey, ez)), eq = group_max<L>(g, c.real ? e : 0);
         const int K2 = 2 * (1040 - eq);                      // velocity changes are in 2^-K2
         const int el = ev - 1023 - K2;
         ok = (unsigned)(eq - 1007) <= 56u && (unsigned)(el + 60) <= 120u;
@@ -847,10 +908,56 @@ __device__ __forceinline__ bool interact_pairs(const Group<L>& g, const Masses<L
         const pairs::Coord Z = pairs::chunks(fixed::to_fixed(bz, 5 + eq - ez));
         pairs::Pair ax = {0.0f, 0.0f}, ay = {0.0f, 0.0f}, az = {0.0f, 0.0f};
         // a term is accepted up to 2^-10 of the velocity, and weaker for
-        // separations where the grid shows (below 2^-7 of its extent)
+        // separations where the grid shows (below 2^-9 of its extent)
         auto accept = [](const pairs::Separation& s, float w, float v) {
             return fmaxf(pairs::mul(w, pairs::mul(s.r2, s.y1)), pairs::mul(w, 256.0f)) <= pairs::mul(v, 1.0f / 1024.0f);
         };
+        if (GRM != 0) {
+            // a_GR(Q) = -6 (G m0)^2 Q / (c^2 |Q|^4); kgr = -6 m0^2 dt / c^2.
+            const pairs::Separation s = pairs::separation(pairs::own(X), pairs::own(Y), pairs::own(Z));
+            const float sc = fixed::bits_to_f32((unsigned)(127 + 1040 - eq) << 23);
+            pairs::Pair k;
+            k.h = pairs::mul(c.kgp.h, sc);
+            k.l = pairs::mul(c.kgp.l, sc);
+            const pairs::Pair w = pairs::product(k, pairs::inverse_fourth(s));
+            const float mf = (float)c.m;
+            const float vg = gr_scale(vl, e, c.jm, K2);
+            ok = ok & accept(s, -w.h, GRM == 1 ? vg : vl);
+            pairs::Pair fx = pairs::product(w, s.x), fy = pairs::product(w, s.y), fz = pairs::product(w, s.z);
+            if (GRM == 2) {                              // minus the mass-weighted sum, on every planet
+                pairs::Pair bx = pairs::product(c.mrp, fx), by = pairs::product(c.mrp, fy), bz = pairs::product(c.mrp, fz);
+                sum_pairs<L>(g, bx, by, bz);
+                if (L == 4 || L == 8) {
+                    const pairs::Pair b = bx;
+                    bx = shfl_pair<L>(b, g.base);
+                    by = shfl_pair<L>(b, g.base + L / 4);
+                    bz = shfl_pair<L>(b, g.base + L / 2);
+                }
+                pairs::accumulate(fx, -bx.h, -bx.l);
+                pairs::accumulate(fy, -by.h, -by.l);
+                pairs::accumulate(fz, -bz.h, -bz.l);
+            }
+            if (GRM == 2) {
+                const float top = fmaxf(fabsf(fx.h), fmaxf(fabsf(fy.h), fabsf(fz.h)));
+                ok = ok & (top <= pairs::mul(vg, 1.0f / 1024.0f));
+            }
+            pairs::accumulate(ax, fx.h, fx.l);
+            pairs::accumulate(ay, fy.h, fy.l);
+            pairs::accumulate(az, fz.h, fz.l);
+            float px = pairs::mul(mf, fx.h), py = pairs::mul(mf, fy.h), pz = pairs::mul(mf, fz.h);
+            sum_floats<L>(g, px, py, pz);
+            double Px, Py, Pz;                           // the second jump
+            if (L == 4 || L == 8) {
+                gather3<L>(g, P.k + pairs::widen(px, K2), Px, Py, Pz);
+            } else {
+                Px = P.x + pairs::widen(px, K2);
+                Py = P.y + pairs::widen(py, K2);
+                Pz = P.z + pairs::widen(pz, K2);
+            }
+            qx = fma(c.jc, Px, qx);
+            qy = fma(c.jc, Py, qy);
+            qz = fma(c.jc, Pz, qz);
+        }
 #pragma unroll
         for (int k = 1; 2 * k <= L; ++k) {
             const int to = g.at(k), from = g.at(-k);
@@ -873,7 +980,7 @@ __device__ __forceinline__ bool interact_pairs(const Group<L>& g, const Masses<L
             if (2 * k < L) {                             // reaction on the partner: -hm_i (Q_j - Q_i)/r^3
                 const pairs::Pair wi = pairs::product(c.hmp, r3);
                 const float vj = __shfl_sync(WHG_FULL_MASK, vl, to);   // (every lane takes part)
-                fit = fit && accept(s, wi.h, vj);
+                fit = fit & accept(s, wi.h, vj);
                 const pairs::Pair gx = pairs::product(wi, s.x), gy = pairs::product(wi, s.y),
                                   gz = pairs::product(wi, s.z);
                 auto take = [&](pairs::Pair& a, const pairs::Pair& f) {
@@ -885,54 +992,12 @@ __device__ __forceinline__ bool interact_pairs(const Group<L>& g, const Masses<L
                 take(az, gz);
             }
             const bool on = (c.pairs_on >> k) & 1u;
-            ok = ok && (fit || !on);
+            ok = ok & (fit | !on);
             if (hill) {
                 const double r2 = pairs::widen(s.r2, -K2);       // by the leading part, where that decides
                 const long long t = __double_as_longlong(thr2[k - 1]), b = __double_as_longlong(r2);
                 if (on && b - (1LL << 32) < t) close |= __double_as_longlong(r2 + pairs::widen(s.r2l, -K2)) < t;
             }
-        }
-        if (GRM != 0) {
-            // a_GR(Q) = -6 (G m0)^2 Q / (c^2 |Q|^4); kgr = -6 m0^2 dt / c^2.
-            const pairs::Separation s = pairs::separation(pairs::own(X), pairs::own(Y), pairs::own(Z));
-            const float sc = fixed::bits_to_f32((unsigned)(127 + 1040 - eq) << 23);
-            pairs::Pair k;
-            k.h = pairs::mul(c.kgp.h, sc);
-            k.l = pairs::mul(c.kgp.l, sc);
-            const pairs::Pair w = pairs::product(k, pairs::inverse_fourth(s));
-            ok = ok && accept(s, -w.h, vl);
-            pairs::Pair fx = pairs::product(w, s.x), fy = pairs::product(w, s.y), fz = pairs::product(w, s.z);
-            if (GRM == 2) {                              // minus the mass-weighted sum, on every planet
-                const float mr = (float)c.mrat;
-                float bx = pairs::mul(mr, fx.h), by = pairs::mul(mr, fy.h), bz = pairs::mul(mr, fz.h);
-                sum_floats<L>(g, bx, by, bz);
-                if (L == 4 || L == 8) {
-                    const float b = bx;
-                    bx = __shfl_sync(WHG_FULL_MASK, b, g.base);
-                    by = __shfl_sync(WHG_FULL_MASK, b, g.base + L / 4);
-                    bz = __shfl_sync(WHG_FULL_MASK, b, g.base + L / 2);
-                }
-                pairs::accumulate(fx, -bx, 0.0f);
-                pairs::accumulate(fy, -by, 0.0f);
-                pairs::accumulate(fz, -bz, 0.0f);
-            }
-            pairs::accumulate(ax, fx.h, fx.l);
-            pairs::accumulate(ay, fy.h, fy.l);
-            pairs::accumulate(az, fz.h, fz.l);
-            const float mf = (float)c.m;
-            float px = pairs::mul(mf, fx.h), py = pairs::mul(mf, fy.h), pz = pairs::mul(mf, fz.h);
-            sum_floats<L>(g, px, py, pz);
-            double Px, Py, Pz;                           // the second jump
-            if (L == 4 || L == 8) {
-                gather3<L>(g, P.k + pairs::widen(px, K2), Px, Py, Pz);
-            } else {
-                Px = P.x + pairs::widen(px, K2);
-                Py = P.y + pairs::widen(py, K2);
-                Pz = P.z + pairs::widen(pz, K2);
-            }
-            qx = fma(c.jc, Px, qx);
-            qy = fma(c.jc, Py, qy);
-            qz = fma(c.jc, Pz, qz);
         }
         vx += pairs::widen(ax.h, K2) + pairs::widen(ax.l, K2);
         vy += pairs::widen(ay.h, K2) + pairs::widen(ay.l, K2);
@@ -1404,12 +1469,13 @@ __device__ __forceinline__ int bucket_of(const WhgBuckets& bk, int w)
     default: { constexpr int L_ = 8; CALL; } break; \
     }
 
-// BLOCKS: blocks of WHG_MAX_BLOCK threads that the register count leaves room for
-// on an SM.  2 (128 registers, 16 resident one-warp blocks) where more than
-// 8 warps per SM share the pipes; 1 (any number of registers, a schedule for
-// one warp's own latency) below.
-template <int NT, int GRM, int BLOCKS>
-__global__ void __launch_bounds__(WHG_MAX_BLOCK, BLOCKS) k_step(WhgState st, WhgBuckets bk, long long n)
+// KIND 2 (160 registers, 12 resident warps) where more than 8 warps per SM share
+// the pipes; 1 (any number of registers, a schedule for one warp's own latency)
+// below.  With 128 registers (16 warps) KIND 2 spilled up to 350 bytes: 2^20
+// 8-planet systems 0.966 ms per step against 0.914, 8192 8.07 us against 7.70,
+// 65,536 compact ones 43.2 us against 39.4; 136 (15 warps) 1.006 ms, 144 (14) 0.930.
+template <int NT, int GRM, int KIND>
+__global__ void __maxnreg__(KIND == 2 ? 160 : 255) k_step(WhgState st, WhgBuckets bk, long long n)
 {
     const int w = warp_index();
     if (w >= bk.warp0[bk.nb]) return;                // whole warps beyond the last bucket
@@ -1449,8 +1515,7 @@ __device__ __noinline__ void queue_unit(const WhgState& st, const WhgBuckets& bk
 }
 
 template <int NT, int GRM>
-__global__ void __launch_bounds__(WHG_MAX_BLOCK, 2) k_step_queue(WhgState st, WhgBuckets bk, long long n,
-                                                             WhgQueue q)
+__global__ void __maxnreg__(160) k_step_queue(WhgState st, WhgBuckets bk, long long n, WhgQueue q)
 {
     const int G = bk.warp0[bk.nb];
     const unsigned long long total = (unsigned long long)G * (unsigned long long)q.units;

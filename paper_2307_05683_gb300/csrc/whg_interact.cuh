@@ -156,6 +156,16 @@ WHG_HD void accumulate(Pair& s, float h, float l)
     s.l = add(s.l, add(t.l, l));
 }
 
+// a + b to ~2^-47 of the larger, the same bits as b + a.
+WHG_HD Pair sum(const Pair& a, const Pair& b)
+{
+    const Pair t = two_sum(a.h, b.h);
+    Pair r;
+    r.h = t.h;
+    r.l = add(t.l, add(a.l, b.l));
+    return r;
+}
+
 // a - b, never contracted with the product that a may be.
 #if defined(__CUDA_ARCH__)
 __device__ __forceinline__ double sub64(double a, double b) { return __dsub_rn(a, b); }

@@ -173,10 +173,10 @@ static int sm_count()
 //   3.61 / 4.19, 2432 (16) 5.54 / 4.19; 5 planets 777 (5) 2.89 / 3.60,
 //   1500 (10) 3.61 / 3.60; 2 planets 4864 (8) 2.49 / 2.89, 9728 (16) 5.25 / 2.94;
 // * one lane per planet, registers for one warp's own chain of instructions
-//   (178; k_step<.., 1>), up to 8 warps per SM;
-// * one lane per planet, 128 registers, above: the resident warps count.  178 /
-//   128 registers: 2432 systems (4 warps per SM) 4.21 / 4.76, 4096 (6.7) 4.82 /
-//   5.33, 8192 (13.5) 9.1 / 7.98.
+//   (187; k_step<.., 1>), up to 8 warps per SM;
+// * one lane per planet, 160 registers, above: the resident warps count.  187 /
+//   160 registers: 2432 systems (4 warps per SM) 4.05 / 4.33, 4096 (6.7) 4.70 /
+//   4.86, 4864 (8) 5.19 / 5.43, 5200 (8.6) 9.70 / 5.67.
 static bool wide_warps(const WhgState& st, const WhgBuckets& bk, int sms)
 {
     if (st.full_rotation) return false;              // interaction schedule without reactions: FP64 only

@@ -93,6 +93,22 @@ __device__ __forceinline__ float wide_sum_float(const WideGroup<L>& g, float x)
     return s;
 }
 
+// sum_pairs of this lane's coordinate.
+template <int L>
+__device__ __forceinline__ pairs::Pair wide_sum_pair(const WideGroup<L>& g, pairs::Pair x)
+{
+    if (L == 1) return x;
+    if (L == 4 || L == 8) {
+#pragma unroll
+        for (int o = L / 2; o; o >>= 1) x = add_xor<L>(x, x, o);
+        return x;
+    }
+    pairs::Pair s = {0.0f, 0.0f};
+#pragma unroll
+    for (int j = 0; j < L; ++j) s = pairs::sum(s, shfl_pair<L>(x, g.in_group ? g.base + j : g.lane));
+    return s;
+}
+
 // interact_pairs on kept coordinates (q, v).  hmk: hm of the partner at the
 // role's distance.
 template <int L, int GRM>
@@ -124,6 +140,31 @@ __device__ __forceinline__ bool wide_interact(const WideGroup<L>& g, const Masse
         auto accept = [](const pairs::Separation& s, float w, float scale) {
             return fmaxf(pairs::mul(w, pairs::mul(s.r2, s.y1)), pairs::mul(w, 256.0f)) <= pairs::mul(scale, 1.0f / 1024.0f);
         };
+        auto gr_kick = [&]() {                           // its terms before those of the pairs, as interact_pairs has them
+            if (GRM == 0) return;
+            const pairs::Pair ox = pairs::own(X), oy = pairs::own(Y), oz = pairs::own(Z);
+            const pairs::Separation s = pairs::separation(ox, oy, oz);
+            const float sc = fixed::bits_to_f32((unsigned)(127 + 1040 - eq) << 23);
+            pairs::Pair k;
+            k.h = pairs::mul(c.kgp.h, sc);
+            k.l = pairs::mul(c.kgp.l, sc);
+            const pairs::Pair w = pairs::product(k, pairs::inverse_fourth(s));
+            const float mf = (float)c.m, vg = gr_scale(vl, (int)(top >> 16), c.jm, K2);
+            ok = ok & accept(s, -w.h, GRM == 1 ? vg : vl);
+            pairs::Pair o;
+            o.h = g.mine(ox.h, oy.h, oz.h);
+            o.l = g.mine(ox.l, oy.l, oz.l);
+            pairs::Pair f = pairs::product(w, o);
+            if (GRM == 2) {
+                const pairs::Pair b = wide_sum_pair<L>(g, pairs::product(c.mrp, f));
+                pairs::accumulate(f, -b.h, -b.l);
+                ok = ok & (fabsf(f.h) <= pairs::mul(vg, 1.0f / 1024.0f));
+            }
+            pairs::accumulate(a, f.h, f.l);
+            const float p = wide_sum_float<L>(g, pairs::mul(mf, f.h));
+            q = fma(c.jc, P + pairs::widen(p, K2), q);
+        };
+        if (L == 1) gr_kick();
         if (L > 1) {
             const int k = 2 * (g.r + 1) <= L ? g.r + 1 : 1;      // this role's distance (roles beyond L/2 idle along)
             auto at = [&](const pairs::Coord& x, int j) {
@@ -140,11 +181,11 @@ __device__ __forceinline__ bool wide_interact(const WideGroup<L>& g, const Masse
             const pairs::Pair r3 = pairs::inverse_cube(s);
             const pairs::Pair wj = pairs::product(hmk, r3), wi = pairs::product(c.hmp, r3);
             const float vj = __shfl_sync(WHG_FULL_MASK, vl, g.lane_of(g.r, k));
-            const bool fit = accept(s, wj.h, vl) && (2 * k == L || accept(s, wi.h, vj));
+            const bool fit = accept(s, wj.h, vl) & ((2 * k == L) | accept(s, wi.h, vj));
             const pairs::Pair fx = pairs::product(wj, s.x), fy = pairs::product(wj, s.y), fz = pairs::product(wj, s.z);
             const pairs::Pair gx = pairs::product(wi, s.x), gy = pairs::product(wi, s.y), gz = pairs::product(wi, s.z);
-            const bool on = g.r == k - 1 && ((c.pairs_on >> k) & 1u);
-            ok = ok && (fit || !on);
+            const bool on = (g.r == k - 1) & ((c.pairs_on >> k) & 1u);
+            ok = ok & (fit | !on);
             if (hill) {
                 const double r2 = pairs::widen(s.r2, -K2);       // by the leading part, where that decides
                 const double t2 = k == 1 ? thr2[0] : (k == 2 ? thr2[1] : (k == 3 ? thr2[2] : thr2[3]));
@@ -156,6 +197,7 @@ __device__ __forceinline__ bool wide_interact(const WideGroup<L>& g, const Masse
                             sz = __shfl_sync(WHG_FULL_MASK, z, lane);
                 return g.mine(sx, sy, sz);
             };
+            gr_kick();
 #pragma unroll
             for (int d = 1; 2 * d <= L; ++d) {                   // in step_body's order
                 const int own = g.lane_of(d - 1, 0);
@@ -167,27 +209,6 @@ __device__ __forceinline__ bool wide_interact(const WideGroup<L>& g, const Masse
                     pairs::accumulate(a, -bh, -bl);
                 }
             }
-        }
-        if (GRM != 0) {
-            const pairs::Pair ox = pairs::own(X), oy = pairs::own(Y), oz = pairs::own(Z);
-            const pairs::Separation s = pairs::separation(ox, oy, oz);
-            const float sc = fixed::bits_to_f32((unsigned)(127 + 1040 - eq) << 23);
-            pairs::Pair k;
-            k.h = pairs::mul(c.kgp.h, sc);
-            k.l = pairs::mul(c.kgp.l, sc);
-            const pairs::Pair w = pairs::product(k, pairs::inverse_fourth(s));
-            ok = ok && accept(s, -w.h, vl);
-            pairs::Pair o;
-            o.h = g.mine(ox.h, oy.h, oz.h);
-            o.l = g.mine(ox.l, oy.l, oz.l);
-            pairs::Pair f = pairs::product(w, o);
-            if (GRM == 2) {
-                const float b = wide_sum_float<L>(g, pairs::mul((float)c.mrat, f.h));
-                pairs::accumulate(f, -b, 0.0f);
-            }
-            pairs::accumulate(a, f.h, f.l);
-            const float p = wide_sum_float<L>(g, pairs::mul((float)c.m, f.h));
-            q = fma(c.jc, P + pairs::widen(p, K2), q);
         }
         v += pairs::widen(a.h, K2) + pairs::widen(a.l, K2);
     }
