@@ -252,6 +252,40 @@ __device__ __forceinline__ double rsqrt_pow(double x)
 __device__ __forceinline__ double rsqrt(double x) { return rsqrt_pow<false>(x); }
 __device__ __forceinline__ double rsqrt_cubed(double x) { return rsqrt_pow<true>(x); }
 
+// FP64 -> FP32 from the bit fields (sign, exponent rebiased from 1023 to
+// 127, mantissa truncated to 23 bits) on the integer pipe: the hardware
+// conversion runs on the FP64 pipe, the scarce unit here.  Rounds toward
+// zero; |x| below the FP32 normal range gives a signed zero, above it (and
+// inf, NaN) a signed infinity.
+__device__ __forceinline__ float to_f32(double x)
+{
+    const unsigned hi = (unsigned)__double2hiint(x);
+    const unsigned lo = (unsigned)__double2loint(x);
+    const unsigned sign = hi & 0x80000000u;
+    const int ex = (int)((hi >> 20) & 0x7ffu) - 1023 + 127;            // FP32 biased exponent
+    unsigned b = sign | ((unsigned)ex << 23) | ((hi & 0x000fffffu) << 3) | (lo >> 29);
+    b = ex <= 0 ? sign : b;
+    b = ex >= 255 ? (sign | 0x7f800000u) : b;
+    return __uint_as_float(b);
+}
+
+// FP32 -> FP64 from the bit fields (exact for normal numbers; subnormals give
+// a signed zero; inf and NaN stay inf and NaN), on the integer pipe.
+__device__ __forceinline__ double to_f64(float f)
+{
+    const unsigned b = __float_as_uint(f);
+    const unsigned sign = b & 0x80000000u;
+    const unsigned ex = (b >> 23) & 0xffu;
+    const unsigned man = b & 0x007fffffu;
+    unsigned hi = sign | ((ex + 896u) << 20) | (man >> 3);
+    unsigned lo = man << 29;
+    hi = ex == 0u ? sign : hi;
+    lo = ex == 0u ? 0u : lo;
+    hi = ex == 255u ? (sign | 0x7ff00000u | (man ? 0x00080000u : 0u)) : hi;
+    lo = ex == 255u ? 0u : lo;
+    return __hiloint2double((int)hi, (int)lo);
+}
+
 __device__ __forceinline__ bool is_finite(double x)
 {
     return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000;
@@ -306,11 +340,12 @@ __device__ __forceinline__ void stumpff_c2c3(double z, double& c2, double& c3)
 // (the second forms use G0 = 1 - beta G2, G1 = X - beta G3 and
 // zeta0 = mu - beta r0, so only the c2 and c3 series are needed): initial
 // guess h/r0 (the first-order value of X(h); the paper gives none), 2 Halley
-// steps with 4-term series, 2 Newton steps with NT-term series.  The G_n at
+// steps with 4-term series, 2 Newton steps with NT-term series.  The Halley steps
+// run in FP32 where that holds them (general_start), else in FP64.  The G_n at
 // the final X = X1 + d come from the values at the last Newton point X1 by
 // one Taylor step (dG_n/dX = G_{n-1}); |d| is the last Newton correction, so
 // the neglected d^2 terms are far below rounding.  Then the Lagrange f - 1,
-// g, fdot, gdot - 1.  No branches.
+// g, fdot, gdot - 1.  r0sq, eta0 and v2 are Q.Q, Q.v and v.v.
 // Returns beta > 0.  With VALS, *dv also receives the drift's intermediate
 // values (for the adjoint's tape); the arithmetic is the same either way.
 struct DriftVals {
@@ -320,22 +355,35 @@ struct DriftVals {
     double ri, A, fm1, g, fd, gdm1;      // 1/r, mu/r0, Lagrange coefficients
 };
 
-template <int NT, bool VALS>
-__device__ __forceinline__ bool kepler_general(double mu, double h, double& qx, double& qy,
-                                             double& qz, double& vx, double& vy, double& vz,
-                                             DriftVals* dv)
+// The two Halley steps in FP32, as s = X r0/h from s = 1; 0 where they are not to
+// be used: unbound orbits, mu h^2/r0^3 >= 4096 or outside FP32, a result that is
+// no start.  They only supply the Newton steps' start: where the step resolves
+// the pericentre (a pericentre timescale of two steps or more, mu h^2/r0^3 < 10)
+// the FP32 rounding, ~1e-6 of s, is below what two Halley steps leave at that limit
+// (1e-4), and two Newton steps square either twice.
+__device__ __forceinline__ float general_start(double mu, double h, double r0i, double eta0, double v2)
 {
-    const double r0sq = fma(qx, qx, fma(qy, qy, qz * qz));
+    using fixed::mul;
+    const float rf = to_f32(r0i), w = mul(to_f32(h), rf), w2 = mul(w, w);
+    const float a = mul(mul(to_f32(eta0), rf), w), m = mul(mul(to_f32(mu), rf), w2), V = mul(to_f32(v2), w2);
+    if (!(V < 2.0f * m && m < 4096.0f)) return 0.0f;
+    const float s = fixed::halley(1.0f, a, fixed::sub(V, m), fixed::fma(2.0f, m, -V));
+    return s > 0x1p-10f && s < 0x1p10f ? s : 0.0f;
+}
+
+template <int NT, bool VALS>
+__device__ __forceinline__ bool kepler_general(double mu, double h, double r0sq, double eta0, double v2, double& qx,
+                                               double& qy, double& qz, double& vx, double& vy, double& vz, DriftVals* dv)
+{
     const double r0i = rsqrt(r0sq);
     const double r0 = r0sq * r0i;
-    const double eta0 = fma(qx, vx, fma(qy, vy, qz * vz));
-    const double v2 = fma(vx, vx, fma(vy, vy, vz * vz));
     const double beta = fma(2.0 * mu, r0i, -v2);
     const double zeta0 = fma(-beta, r0, mu);
-    double X, X2, c2, c3, G1, G2, G3;
-    X = h * r0i;
+    double X = h * r0i, X2, c2, c3, G1, G2, G3;
+    const float s = general_start(mu, h, r0i, eta0, v2);
+    if (s > 0.0f) X *= to_f64(s);
 #pragma unroll
-    for (int it = 0; it < 2; ++it) {             // Halley
+    for (int it = 0; it < 2 && !(s > 0.0f); ++it) {      // Halley
         X2 = X * X;
         stumpff_c2c3<4>(beta * X2, c2, c3);
         G2 = X2 * c2;
@@ -359,7 +407,7 @@ __device__ __forceinline__ bool kepler_general(double mu, double h, double& qx, 
         const double F = fma(r0, X, fma(eta0, G2, fma(zeta0, G3, -h)));
         const double Fp = fma(zeta0, G2, fma(eta0, G1, r0));
         if (it == 0) X = fma(-F, rcp(Fp), X);        // the first correction applied at once
-        else d = -F * rcp(Fp);                       // the last one kept for the G_n update
+        else d = __dmul_rn(-F, rcp(Fp));             // the last one kept for the G_n update
     }
     // G at the final X + d from the last Newton point X.
     const double G0 = fma(-beta, G2, 1.0);
@@ -390,8 +438,8 @@ __device__ __forceinline__ bool kepler_general(double mu, double h, double& qx, 
     return beta > 0.0;
 }
 
-// kepler_general as one out-of-line function for all callers: it is rarely
-// run, and inlined it would hold registers and code of every step kernel.
+// kepler_general as one out-of-line function for all callers: few states need
+// it, and inlined it would hold registers and code of every step kernel.
 template <bool VALS>
 struct GeneralDrift {
     double qx, qy, qz, vx, vy, vz;
@@ -405,12 +453,13 @@ struct GeneralDrift<false> {
 };
 
 template <int NT, bool VALS>
-__device__ __noinline__ GeneralDrift<VALS> kepler_general_call(double mu, double h, double qx, double qy, double qz,
-                                                               double vx, double vy, double vz)
+__device__ __noinline__ GeneralDrift<VALS> kepler_general_call(double mu, double h, double r0sq, double eta0, double v2,
+                                                               double qx, double qy, double qz, double vx, double vy,
+                                                               double vz)
 {
     GeneralDrift<VALS> r;
     DriftVals dv;
-    r.bound = kepler_general<NT, VALS>(mu, h, qx, qy, qz, vx, vy, vz, &dv);
+    r.bound = kepler_general<NT, VALS>(mu, h, r0sq, eta0, v2, qx, qy, qz, vx, vy, vz, &dv);
     r.qx = qx; r.qy = qy; r.qz = qz;
     r.vx = vx; r.vy = vy; r.vz = vz;
     if constexpr (VALS) r.dv = dv;
@@ -418,10 +467,19 @@ __device__ __noinline__ GeneralDrift<VALS> kepler_general_call(double mu, double
 }
 
 // The drift: the solution of Kepler's equation in fixed point (whg_fixed.cuh)
-// inside that solver's domain, which holds every resolved bound orbit, else
-// kepler_general.  The choice depends on the planet's own state only, so
-// results do not depend on which lane or warp holds it.  21 FP64
-// instructions (three scalar products and the new vectors) against 153.
+// inside that solver's domain, else kepler_general.  The choice depends on the
+// planet's own state only, so results do not depend on which lane or warp
+// holds it.  21 FP64 instructions (three scalar products and the new vectors)
+// against 153.
+//
+// A warp with a planet on each side runs both solvers one after the other, so the
+// general one must cost less than the FP64 pipe time that the other saves.  It
+// does from its FP32 start: 93 FP64 instructions, 147 with the Halley steps in
+// FP64.  5-day steps, us per step with every solver step in FP64 / both solvers,
+// Halley in FP64 / in FP32: 20,000 particles at a = 0.387, e = 0.7 (6.7 % of the
+// phases outside the domain) 7.47 / 8.48 / 6.15, e = 0.8 7.47 / 9.29 / 6.65, e = 0.6
+// (none outside) 7.47 / 2.60 / 2.60; 200,000 of a = 0.1 to 1, e up to 0.95 59.5 /
+// 63.8 / 43.5; 100 of them 5.84 / 7.02 / 5.10.
 template <int NT, bool VALS = false>
 __device__ __forceinline__ bool kepler_drift(double mu, double h, double& qx, double& qy, double& qz, double& vx,
                                              double& vy, double& vz, DriftVals* dv = nullptr, bool live = true)
@@ -432,7 +490,7 @@ __device__ __forceinline__ bool kepler_drift(double mu, double h, double& qx, do
     fixed::Solution o;
     if (!fixed::solve<NT, VALS>(mu, h, r0sq, eta0, v2, o)) {
         if (!live) return false;
-        const GeneralDrift<VALS> r = kepler_general_call<NT, VALS>(mu, h, qx, qy, qz, vx, vy, vz);
+        const GeneralDrift<VALS> r = kepler_general_call<NT, VALS>(mu, h, r0sq, eta0, v2, qx, qy, qz, vx, vy, vz);
         qx = r.qx; qy = r.qy; qz = r.qz;
         vx = r.vx; vy = r.vy; vz = r.vz;
         if constexpr (VALS) *dv = r.dv;

@@ -193,40 +193,6 @@ __device__ double rsqrt_cubed_fp64_ref(double x)
     return fma(y3 * e, fma(1.875, e, 1.5), y3);
 }
 
-// FP64 -> FP32 from the bit fields (sign, exponent rebiased from 1023 to
-// 127, mantissa truncated to 23 bits) on the integer pipe: the hardware
-// conversion runs on the FP64 pipe, the scarce unit here.  Rounds toward
-// zero; |x| below the FP32 normal range gives a signed zero, above it (and
-// inf, NaN) a signed infinity.
-__device__ __forceinline__ float to_f32(double x)
-{
-    const unsigned hi = (unsigned)__double2hiint(x);
-    const unsigned lo = (unsigned)__double2loint(x);
-    const unsigned sign = hi & 0x80000000u;
-    const int ex = (int)((hi >> 20) & 0x7ffu) - 1023 + 127;            // FP32 biased exponent
-    unsigned b = sign | ((unsigned)ex << 23) | ((hi & 0x000fffffu) << 3) | (lo >> 29);
-    b = ex <= 0 ? sign : b;
-    b = ex >= 255 ? (sign | 0x7f800000u) : b;
-    return __uint_as_float(b);
-}
-
-// FP32 -> FP64 from the bit fields (exact for normal numbers; subnormals give
-// a signed zero; inf and NaN stay inf and NaN), on the integer pipe.
-__device__ __forceinline__ double to_f64(float f)
-{
-    const unsigned b = __float_as_uint(f);
-    const unsigned sign = b & 0x80000000u;
-    const unsigned ex = (b >> 23) & 0xffu;
-    const unsigned man = b & 0x007fffffu;
-    unsigned hi = sign | ((ex + 896u) << 20) | (man >> 3);
-    unsigned lo = man << 29;
-    hi = ex == 0u ? sign : hi;
-    lo = ex == 0u ? 0u : lo;
-    hi = ex == 255u ? (sign | 0x7ff00000u | (man ? 0x00080000u : 0u)) : hi;
-    lo = ex == 255u ? 0u : lo;
-    return __hiloint2double((int)hi, (int)lo);
-}
-
 __global__ void k_special(const double* x, int n, double* out)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -237,7 +203,7 @@ __global__ void k_special(const double* x, int n, double* out)
     out[n + i] = 1.0 / v;
     out[2 * n + i] = pos ? whg::rsqrt(v) : 0.0;
     out[3 * n + i] = pos ? ::rsqrt(v) : 0.0;
-    out[4 * n + i] = to_f64(to_f32(v));
+    out[4 * n + i] = whg::to_f64(whg::to_f32(v));
     out[5 * n + i] = (double)__double2float_rz(v);
     out[6 * n + i] = rcp_fp64_ref(v);
     out[7 * n + i] = pos ? rsqrt_fp64_ref(v) : 0.0;

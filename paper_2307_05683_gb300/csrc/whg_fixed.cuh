@@ -243,11 +243,9 @@ WHG_HD void stumpff(u64 x, u64& c2, u64& c3)
     c3 = coef(0, 3, 65) - mulhi(x, p3);
 }
 
-// Two Halley steps in FP32 for phi(s) = 0.
-WHG_HD float start(float a, float b, float B)
+// Two Halley steps in FP32 for phi(s) = 0, from s.
+WHG_HD float halley(float s, float a, float b, float B)
 {
-    float s = fma(-1.0f / 6.0f, b, fma(0.5f, fma(a, a, -a), 1.0f));
-    s = s < 0.6f ? 0.6f : (s > 1.7f ? 1.7f : s);
 #if defined(__CUDA_ARCH__)
 #pragma unroll
 #endif
@@ -269,6 +267,12 @@ WHG_HD float start(float a, float b, float B)
         s = fma(-mul(F, R), rcp_f32(fma(R, R, mul(-0.5f, mul(F, R1)))), s);
     }
     return s;
+}
+
+WHG_HD float start(float a, float b, float B)
+{
+    const float s = fma(-1.0f / 6.0f, b, fma(0.5f, fma(a, a, -a), 1.0f));
+    return halley(s < 0.6f ? 0.6f : (s > 1.7f ? 1.7f : s), a, b, B);
 }
 
 struct Solution {

@@ -278,7 +278,7 @@ __device__ __forceinline__ void wide_body(const WhgState& st, const WhgBuckets& 
             v = fma(-o.fdn, q, fma(-o.gdm1n, v, v));
             q = nq;
         } else if (alive) {
-            const GeneralDrift<false> r = kepler_general_call<NT, false>(mu, hK, qx, qy, qz, vx, vy, vz);
+            const GeneralDrift<false> r = kepler_general_call<NT, false>(mu, hK, r0sq, eta0, v2, qx, qy, qz, vx, vy, vz);
             q = g.mine(r.qx, r.qy, r.qz);
             v = g.mine(r.vx, r.vy, r.vz);
             bound = r.bound;
