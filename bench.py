@@ -7,8 +7,8 @@ e and i perturbed by Rayleigh(1e-3), angles seeded), dt = P_Mercury / 20, GR
 term on.  One benchmark step = one whg_step call advancing every system by
 --chunk integrator steps (default 1e4; 100 benchmark steps = the full 1e6
 steps).  The state lives in registers during a launch, so there is no
-per-step memory traffic to cache (with the default work queue it is reloaded
-from L2 every 100 steps); L2 is flushed (256 MB write) between timed steps
+per-step memory traffic to cache (above 8 warps per SM, 4864 systems, the work
+queue reloads it from L2 every 100 steps); L2 is flushed (256 MB write) between timed steps
 anyway.
 
 Prints ONE JSON line.  --impl reference times the CPU oracle instead (rank 0).
@@ -46,18 +46,28 @@ UNIT = "system-steps/s"
 # table equal to the oracle's count.
 ALG_FLOPS = {(8, 8, 1): 3464, (8, 8, 0): 3336, (8, 6, 1): 3272, (8, 8, 2): 3536}
 # Of these, the Kepler solver's starting phase (initial guess and the two
-# Halley steps, 8 drifts): with the halley_fp32 option they run on the FP32
-# pipe, and that option's FP64 roofline counts ALG_FLOPS - START_FLOPS.
+# Halley steps, 8 drifts), which the library runs in FP32.
 START_FLOPS = {(8, 8, 1): 776, (8, 8, 0): 776, (8, 6, 1): 776, (8, 8, 2): 776}
 # The same count for systems of n = 1..8 planets (8-term series, GR on), for
 # ensembles of mixed planet counts; a CPU test keeps it equal to the oracle's.
 ALG_FLOPS_BY_PLANETS = {1: 349, 2: 722, 3: 1119, 4: 1540, 5: 1985, 6: 2454, 7: 2947, 8: 3464}
 
 
-# Flops of one system-step that run on the FP64 pipe, FMA = 2 (ncu on the bench
-# launch: 208 FMA, 72 additions, 40 products); the rest of the algorithm runs on
-# the integer and FP32 pipes.
+# Flops of one system-step that run on the FP64 pipe, FMA = 2 (ncu on the default
+# launch: 208 FMA, 72 additions, 40 products), in the kernels of one lane per
+# planet with gr_mode 1; the rest of the algorithm runs on the integer and FP32
+# pipes.
 FP64_PIPE_FLOPS = 528
+
+
+def step_kernel(systems: int, gr_mode: int, sms: int = 152) -> tuple[str, int | None]:
+    """The step kernel that an ensemble of 8-planet systems runs (four systems per
+    warp of one-lane kernels, one of the four-lane kernel), and its FP64-pipe flops
+    per system-step where they were counted."""
+    if systems <= 12 * sms:
+        return f"k_step_wide<8,{gr_mode}>", None
+    name = f"k_step<8,{gr_mode},1>" if -(-systems // 4) <= 8 * sms else f"k_step_queue<8,{gr_mode}>"
+    return name, FP64_PIPE_FLOPS if gr_mode == 1 else None
 
 
 def fp64_flops(gr_mode: int, halley_fp32: bool, newton_terms: int = 8) -> int:
@@ -404,19 +414,6 @@ def throughput_sweep(whg, torch, sizes=tuple(1 << k for k in range(14, 21)), win
     return out
 
 
-def solver_comparison(whg, torch, ens, gr_mode: int, window_s=1.0):
-    """The bench workload with and without the halley_fp32 option (which has no
-    effect any more), same timing method."""
-    stream = torch.cuda.Stream()
-    out = {}
-    for h32 in (False, True):
-        rate, n = time_rate(whg, torch, ens, window_s, stream, gr_mode=gr_mode, halley_fp32=h32)
-        out["halley_fp32" if h32 else "default"] = {"system_steps_per_s": round(rate, 1), "steps": n}
-    return out
-
-
-# ------------------------------------------------------------ GPU arm --
-
 def run_whg(args):
     import torch
     from paper_2307_05683_gb300 import build, whg
@@ -507,16 +504,17 @@ def run_whg(args):
     flops = fp64_flops(args.gr_mode, False)
     kernel_ms = total_ms / args.steps / max(launches_per_step, 1.0)
     kernel_rate = S * (chunk / max(launches_per_step, 1.0)) / (kernel_ms / 1e3)
-    achieved = FP64_PIPE_FLOPS * kernel_rate / 1e12
+    kernel, pipe_flops = step_kernel(S, args.gr_mode)
+    achieved = pipe_flops * kernel_rate / 1e12 if pipe_flops else None
     adjoint = measure_adjoint(whg, torch) if world == 1 else None
     sweep = throughput_sweep(whg, torch) if world == 1 else None
-    solvers = solver_comparison(whg, torch, ens, args.gr_mode) if world == 1 else None
     uneven = measure_uneven(whg, torch) if world == 1 else None
-    roofline = {"bound": "alu", "achieved": round(achieved, 4), "peak": round(FP64_PEAK_TFLOPS, 4),
-                "unit": "TFLOP/s", "frac": round(achieved / FP64_PEAK_TFLOPS, 4),
+    roofline = {"bound": "alu", "achieved": round(achieved, 4) if achieved else None,
+                "peak": round(FP64_PEAK_TFLOPS, 4), "unit": "TFLOP/s",
+                "frac": round(achieved / FP64_PEAK_TFLOPS, 4) if achieved else None,
                 "traffic": profiled_traffic(),
-                "kernel": "k_step<8,1,1>",
-                "fp64_pipe_flops_per_system_step": FP64_PIPE_FLOPS,
+                "kernel": kernel,
+                "fp64_pipe_flops_per_system_step": pipe_flops,
                 "algorithmic_flops_per_system_step": flops,
                 "algorithmic_tflops": round(flops * kernel_rate / 1e12, 4),
                 "peak_basis": "recipe unit counts x clocks: 152 SMs x 2 FP64 FMA/clk x 2 x 2.07 GHz"}
@@ -532,7 +530,6 @@ def run_whg(args):
             "gpu_launches": int(launches),
             "adjoint": adjoint,
             "sweep": sweep,
-            "solver_comparison": solvers,
             "uneven_batch": uneven,
             "clocks": clock_info,
             "systems_flagged": bad}
