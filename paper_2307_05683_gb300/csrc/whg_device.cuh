@@ -810,7 +810,10 @@ __device__ __forceinline__ Masses<L> masses_of(const Group<L>& g, bool real, dou
 }
 
 // The sub-step in FP64, for the systems that the float-pair form leaves out
-// (and the interaction schedule without reactions).  Out of line: rarely run.
+// (and the interaction schedule without reactions).  Out of line: few systems
+// need it, but their warp runs both forms, and where a launch has one warp per
+// sub-partition it waits for such a warp (4096 compact systems at steps of P/7, four
+// of them redone each step: 17.6 us per step against 11.9 at P/20).
 // Warp shuffles inside: every lane calls it.
 struct SubStep {
     double m, hm, mrat, jc, kgr;
@@ -1038,7 +1041,7 @@ __device__ __forceinline__ bool interact_pairs(const Group<L>& g, const Masses<L
             if (2 * k < L) {                             // reaction on the partner: -hm_i (Q_j - Q_i)/r^3
                 const pairs::Pair wi = pairs::product(c.hmp, r3);
                 const float vj = __shfl_sync(WHG_FULL_MASK, vl, to);   // (every lane takes part)
-                fit = fit & accept(s, wi.h, vj);
+                fit = fit && accept(s, wi.h, vj);
                 const pairs::Pair gx = pairs::product(wi, s.x), gy = pairs::product(wi, s.y),
                                   gz = pairs::product(wi, s.z);
                 auto take = [&](pairs::Pair& a, const pairs::Pair& f) {
@@ -1050,7 +1053,7 @@ __device__ __forceinline__ bool interact_pairs(const Group<L>& g, const Masses<L
                 take(az, gz);
             }
             const bool on = (c.pairs_on >> k) & 1u;
-            ok = ok & (fit | !on);
+            ok = ok && (fit || !on);
             if (hill) {
                 const double r2 = pairs::widen(s.r2, -K2);       // by the leading part, where that decides
                 const long long t = __double_as_longlong(thr2[k - 1]), b = __double_as_longlong(r2);
@@ -1527,13 +1530,15 @@ __device__ __forceinline__ int bucket_of(const WhgBuckets& bk, int w)
     default: { constexpr int L_ = 8; CALL; } break; \
     }
 
-// KIND 2 (160 registers, 12 resident warps) where more than 8 warps per SM share
-// the pipes; 1 (any number of registers, a schedule for one warp's own latency)
-// below.  With 128 registers (16 warps) KIND 2 spilled up to 350 bytes: 2^20
-// 8-planet systems 0.966 ms per step against 0.914, 8192 8.07 us against 7.70,
-// 65,536 compact ones 43.2 us against 39.4; 136 (15 warps) 1.006 ms, 144 (14) 0.930.
-template <int NT, int GRM, int KIND>
-__global__ void __maxnreg__(KIND == 2 ? 160 : 255) k_step(WhgState st, WhgBuckets bk, long long n)
+// BLOCKS: blocks of WHG_MAX_BLOCK threads that the register count leaves room for
+// on an SM.  2 (128 registers, 16 resident one-warp blocks) where more than
+// 8 warps per SM share the pipes; 1 (any number of registers, a schedule for
+// one warp's own latency) below.
+// (160 registers, 12 resident warps, no spills: 1 to 5 % faster where the warps
+// come in many waves or fit in 12 an SM, but 8192 8-planet systems, 13.5 an SM, take
+// two waves: 9.65 us per step against 7.99 in launches without the queue.)
+template <int NT, int GRM, int BLOCKS>
+__global__ void __launch_bounds__(WHG_MAX_BLOCK, BLOCKS) k_step(WhgState st, WhgBuckets bk, long long n)
 {
     const int w = warp_index();
     if (w >= bk.warp0[bk.nb]) return;                // whole warps beyond the last bucket
@@ -1573,7 +1578,7 @@ __device__ __noinline__ void queue_unit(const WhgState& st, const WhgBuckets& bk
 }
 
 template <int NT, int GRM>
-__global__ void __maxnreg__(160) k_step_queue(WhgState st, WhgBuckets bk, long long n, WhgQueue q)
+__global__ void __launch_bounds__(WHG_MAX_BLOCK, 2) k_step_queue(WhgState st, WhgBuckets bk, long long n, WhgQueue q)
 {
     const int G = bk.warp0[bk.nb];
     const unsigned long long total = (unsigned long long)G * (unsigned long long)q.units;
