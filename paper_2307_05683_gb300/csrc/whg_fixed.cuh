@@ -34,7 +34,7 @@
 // With the series cut at z^T, dg_3/ds = g_2 and dg_1/ds = g_0 still hold, but
 // dg_2/ds = g_1 + tau, tau = z^(T+1) s/(2T+3)!.  For T = 8 tau d is below 2^-67;
 // for T = 6 it reaches 2^-53 (z = 2), always of one sign, so G_2 and the step
-// (slope R + a tau) take it along: without, 1 - f and 1 - gdot were off by
+// (slope R + a tau) take it along, tau in FP32: without, 1 - f and 1 - gdot were off by
 // -0.9 2^-53 in the mean for 1.75 < z < 2, with it by -0.03 2^-53, as everywhere.
 //
 // The result's error is ~2^-58 (of h for g, which at the domain's edge is up to
@@ -356,7 +356,8 @@ WHG_HD bool solve(double mu, double h, double r0sq, double eta0, double v2, Solu
     Bs = Bs < 0 ? 0 : Bs;
     const u64 B = (u64)Bs << 1;                                          // Q62
     const float sf = start(af, bf, Bf);
-    if (!(sf > 0.5625f && sf < 1.75f && mul(Bf, mul(sf, sf)) < 1.99f)) return false;
+    const float zf = mul(Bf, mul(sf, sf));
+    if (!(sf > 0.5625f && sf < 1.75f && zf < 1.99f)) return false;
     const u32 sh = f32_to_u32(mul(sf, 1073741824.0f)) - 724u;                // Q30, 2^-20.5 low
 
     // series and g_n at the start
@@ -372,7 +373,14 @@ WHG_HD bool solve(double mu, double h, double r0sq, double eta0, double v2, Solu
 
     // phi (Q60, <= 0 at the low start) and R (Q60)
     const i64 nphi = (i64)(one60 - ((u64)sh << 30) - (mulhi(a1, g2w) - g2) - (mulhi(b2, g3w) - g3));
-    const u64 R = one60 + (mulhi(a1, g1) - (g1 >> 2)) + ((mulhi(b2, g2w) - g2) << 1);
+    u64 R = one60 + (mulhi(a1, g1) - (g1 >> 2)) + ((mulhi(b2, g2w) - g2) << 1);
+    const i32 ah = (i32)hi32(a1) - (i32)(1u << 30), bh = (i32)hi32(b2) - (i32)(1u << 30);    // Q30, Q29
+    u32 tau = 0;                                                         // Q55
+    if (T == 6) {
+        const float z2 = mul(zf, zf), z4 = mul(z2, z2);
+        tau = f32_to_u32(mul(mul(mul(z4, z2), mul(zf, sf)), (float)(36028797018963968.0 / 1307674368000.0)));
+        R += (u64)((i64)smulhi(ah, (i32)tau) * 128);
+    }
     if (!(nphi >= 0 && nphi < (1ll << 41) && R > (one60 >> 1) + (one60 >> 6) && R < (one60 << 1) - (one60 >> 6)))
         return false;
 
@@ -386,21 +394,12 @@ WHG_HD bool solve(double mu, double h, double r0sq, double eta0, double v2, Solu
     const u32 dh = (u32)(d0 >> 18);                                      // Q44
     const u32 d2 = (u32)(((u64)dh * dh) >> 21);                          // d^2/2, Q68
     const u32 g0h = hi32(g0), g1h = hi32(g1), Bh = hi32(B), yh = hi32(y);   // Q30
-    const i32 ah = (i32)hi32(a1) - (i32)(1u << 30), bh = (i32)hi32(b2) - (i32)(1u << 30);    // Q30, Q29
     const i32 R1 = smulhi(ah, (i32)g0h) + 2 * smulhi(bh, (i32)g1h);      // dR/ds, Q28
-    u64 d = d0 - (u64)(i64)smulhi(smulhi(R1, (i32)yh), (i32)d2);
-    u64 dtau = 0;                                                        // d tau, Q60
-    if (T == 6) {
-        const u32 xh = hi32(x), x2 = umulhi(xh, xh), x3 = umulhi(x2, xh);
-        const u32 tau = umulhi(umulhi(umulhi(umulhi(x3, x3), xh), (u32)coef(7, 15, 57)), sh);   // Q55
-        const u64 e = (u64)dh * tau;                                     // Q99
-        dtau = e >> 39;
-        d -= (u64)(((i64)(e >> 37) * smulhi(ah, (i32)yh)) >> 28);
-    }
+    const u64 d = d0 - (u64)(i64)smulhi(smulhi(R1, (i32)yh), (i32)d2);
 
     // g_n at s + d (mulhi's constants also make up for the truncated shifts)
     const u64 G3 = g3 + (mulhi<0x100000000ull>(d, g2w) << 1) + (umulhi(d2, g1h) >> 5);   // Q61
-    const u64 G2 = g2 + mulhi<0x140000000ull>(d, g1) + (umulhi(d2, g0h) >> 6) + dtau;    // Q60
+    const u64 G2 = g2 + mulhi<0x140000000ull>(d, g1) + (umulhi(d2, g0h) >> 6) + (umulhi(dh, tau) >> 7);   // Q60
     const u64 G1 = g1 + (mulhi(d, g0) << 2) - (umulhi(d2, umulhi(Bh, g1h)) >> 2);            // Q62
     const u64 G2w = G2 << 2;
     const u64 Rn = one60 + (mulhi<0xA0000000ull>(a1, G1) - (G1 >> 2)) + ((mulhi(b2, G2w) - G2) << 1);       // Q60
