@@ -149,7 +149,7 @@ __device__ __forceinline__ bool wide_interact(const WideGroup<L>& g, const Masse
             k.h = pairs::mul(c.kgp.h, sc);
             k.l = pairs::mul(c.kgp.l, sc);
             const pairs::Pair w = pairs::product(k, pairs::inverse_fourth(s));
-            const float mf = (float)c.m, vg = gr_scale(vl, (int)(top >> 16), c.jm, K2);
+            const float vg = gr_scale(vl, (int)(top >> 16), c.jm, K2);
             ok = ok & accept(s, -w.h, GRM == 1 ? vg : vl);
             pairs::Pair o;
             o.h = g.mine(ox.h, oy.h, oz.h);
@@ -161,7 +161,7 @@ __device__ __forceinline__ bool wide_interact(const WideGroup<L>& g, const Masse
                 ok = ok & (fabsf(f.h) <= pairs::mul(vg, 1.0f / 1024.0f));
             }
             pairs::accumulate(a, f.h, f.l);
-            const float p = wide_sum_float<L>(g, pairs::mul(mf, f.h));
+            const float p = wide_sum_float<L>(g, pairs::mul(c.mf, f.h));
             q = fma(c.jc, P + pairs::widen(p, K2), q);
         };
         if (L == 1) gr_kick();
