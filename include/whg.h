@@ -110,7 +110,8 @@ typedef struct {
                                  way: they only supply the starting point, after which one step
                                  in 64-bit fixed point reaches the solution to ~2^-58
                                  (csrc/whg_fixed.cuh).  Outside that solver's domain the
-                                 fixed-iteration solver runs in FP64 throughout. */
+                                 Newton steps run in FP64, and the Halley steps too for unbound
+                                 orbits and steps far longer than a pericentre passage. */
     int repack_frozen;        /* -1 (default): on when a stop rule is on
                                  (close_encounter_hill > 0 or eject_factor > 0), else off.
                                  1: every graph_launches step launches (every 16 without
@@ -262,9 +263,10 @@ int whg_adjoint_backward(whg_ctx* ctx, const double* loss_weight, double* grad_p
  * tape_bytes: tape buffers (K * 592 B per planet lane each, kept until
  *   whg_destroy).  0 (default): three; each segment's tape is recomputed
  *   during the backward half, two segments ahead of the back kernels.
- *   With the split, a budget makes the tapes of the segments already passed
- *   be recomputed during the forward half instead, beside it, into up to one
- *   buffer per segment; the forward half then runs on the back kernels' SMs.
+ *   With the split (automatic or asked for), a budget makes the tapes of the
+ *   segments already passed be recomputed during the forward half instead,
+ *   beside it, into up to one buffer per segment; the forward half then runs
+ *   on the back kernels' SMs.  Unsplit, it has no effect.
  *   -1: as many buffers as fit in half of the free device memory at
  *   whg_adjoint_forward; n > 0: at most n bytes (at least 3 buffers).
  *   Segments without a buffer of their own get their tapes recomputed during

@@ -169,14 +169,14 @@ static int sm_count()
 // * four lanes per planet while its warps, four times as many, stay within 8
 //   per SM (2 per sub-partition), or 12 for systems of 6 or more planets, whose
 //   pair rounds it saves most.  us per step, four lanes / one: 8 planets 608
-//   systems (4 warps per SM) 2.24 / 4.08, 1216 (8) 2.85 / 4.08, 1824 (12)
-//   3.61 / 4.07, 2432 (16) 5.55 / 4.06; 5 planets 777 (5) 2.97 / 3.45,
+//   systems (4 warps per SM) 2.21 / 4.08, 1216 (8) 2.88 / 4.14, 1824 (12)
+//   3.64 / 4.11, 2432 (16) 5.55 / 4.11; 5 planets 777 (5) 2.97 / 3.45,
 //   1500 (10) 3.65 / 3.45; 2 planets 4864 (8) 2.58 / 2.96, 9728 (16) 5.25 / 2.99;
 // * one lane per planet, registers for one warp's own chain of instructions
 //   (188; k_step<.., 1>), up to 8 warps per SM;
 // * one lane per planet, 128 registers, above: the resident warps count.  188 /
-//   128 registers: 2432 systems (4 warps per SM) 4.13 / 4.68, 4096 (6.7) 4.70 /
-//   5.17, 4864 (8) 5.25 / 5.88, 8192 (13.5) 10.2 / 7.97.
+//   128 registers: 2432 systems (4 warps per SM) 4.11 / 4.47, 4096 (6.7) 4.70 /
+//   4.89, 4864 (8) 5.23 / 5.50, 8192 (13.5) 10.2 / 7.37.
 static bool wide_warps(const WhgState& st, const WhgBuckets& bk, int sms)
 {
     if (st.full_rotation) return false;              // interaction schedule without reactions: FP64 only

@@ -12,9 +12,9 @@
 // 14 FP64 instructions per warp and step instead of 41, one pair round
 // instead of L/2.  Every sum keeps step_body's order: the same bits.
 //
-// Measured, us per step, step_body's / this kernel: one 8-planet system 3.96 /
-// 2.19, 608 4.21 / 2.22, ten 2-planet systems 2.70 / 1.86, 100 test particles
-// 2.09 / 1.54; whg_kernels_common.cu has where it stops paying.  168 registers:
+// Measured, us per step, step_body's / this kernel: one 8-planet system 3.84 /
+// 2.18, 608 4.08 / 2.21, ten 2-planet systems 2.70 / 1.85, 100 test particles
+// 2.08 / 1.55; whg_kernels_common.cu has where it stops paying.  168 registers:
 // three warps per sub-partition (with 174, two; 1500 systems 3.58 against 5.60).
 //
 // Lanes: Group<L>'s blocks of L lanes in fours; block 4 j + r is role r of the

@@ -36,7 +36,7 @@ def pericentre_timescale(a, e, mu=1.0):
 
 def accuracy_map(a_values, e_values, n_phases=8, years=10.0, dt_days=5.0, seed=0, halley_fp32=False):
     """Relative a error after `years` of massless particles (production kernel;
-    halley_fp32=True runs the solver's starting phase in FP32).
+    halley_fp32 is passed to the library, where it has no effect).
     Returns (err [na, ne, n_phases], status [na, ne, n_phases])."""
     a_values = np.asarray(a_values, float)
     e_values = np.asarray(e_values, float)
@@ -111,7 +111,7 @@ def solar_copies(n_systems: int, seed: int = 0, dt_days: float = 5.0, perturb_m:
 def energy_error_run(ens, total_steps: int, samples: int = 20, gr_mode: int = 1, **options):
     """Relative energy error |E(t)/E(0) - 1| of every system at `samples`
     evenly spaced times (whg_energy on the synchronized state); `options`
-    go to the Integrator (e.g. halley_fp32=True).
+    go to the Integrator (e.g. newton_terms=6).
     Returns (times [samples], errors [samples, S], status [S])."""
     it = whg.Integrator(ens.n_systems, ens.max_planets, gr_mode=gr_mode, **options)
     it.init(ens)
