@@ -799,7 +799,10 @@ __device__ __forceinline__ Masses<L> masses_of(const Group<L>& g, bool real, dou
     // Conversions run on the FP64 pipe.  The compiler would rather repeat these in
     // every step than hold their results, so it is kept from knowing them: 65,536
     // 8-planet systems 56.0 -> 50.5 us per step, 100,000 single planets 9.5 -> 9.0.
-    asm("" : "+f"(k.mf), "+r"(k.jm), "+f"(k.kgp.h), "+f"(k.kgp.l), "+f"(k.hmp.h), "+f"(k.hmp.l), "+f"(k.mrp.h), "+f"(k.mrp.l));
+    // (Only what the mode uses: m/m0 costs a short launch its FP64 division.)
+    asm("" : "+f"(k.hmp.h), "+f"(k.hmp.l));
+    if (GRM != 0) asm("" : "+f"(k.mf), "+r"(k.jm), "+f"(k.kgp.h), "+f"(k.kgp.l));
+    if (GRM == 2) asm("" : "+f"(k.mrp.h), "+f"(k.mrp.l));
     k.real = real;
     k.full = full;
     k.merged = merged;
