@@ -173,8 +173,8 @@ static int sm_count()
 //   3.64 / 4.11, 2432 (16) 5.55 / 4.11; 5 planets 777 (5) 2.97 / 3.45,
 //   1500 (10) 3.65 / 3.45; 2 planets 4864 (8) 2.58 / 2.96, 9728 (16) 5.25 / 2.99;
 // * one lane per planet, registers for one warp's own chain of instructions
-//   (188; k_step<.., 1>), up to 8 warps per SM;
-// * one lane per planet, 128 registers, above: the resident warps count.  188 /
+//   (182; k_step<.., 1>), up to 8 warps per SM;
+// * one lane per planet, 128 registers, above: the resident warps count.  182 /
 //   128 registers: 2432 systems (4 warps per SM) 4.11 / 4.47, 4096 (6.7) 4.70 /
 //   4.89, 4864 (8) 5.23 / 5.50, 8192 (13.5) 10.2 / 7.37.
 static bool wide_warps(const WhgState& st, const WhgBuckets& bk, int sms)
