@@ -88,7 +88,8 @@ typedef struct {
                                  system gets n warp lanes (8 for n = 7), floor(32/n)
                                  systems per warp, all groups in one launch.  1..8
                                  (>= max_planets): that many lanes for every system */
-    int block_size;           /* CUDA threads per block, 0 = auto (multiple of 32) */
+    int block_size;           /* CUDA threads per block (multiple of 32); 0 = auto: 32, or for the
+                                 steps of ensembles with several planet counts up to 256 */
     long long steps_per_launch; /* 0 = auto; bounds one kernel launch's length */
     double close_encounter_hill; /* ensemble stop rule (not in the paper's map), 0 = off:
                                  stop a system when a pair comes closer than this many
@@ -136,7 +137,8 @@ typedef struct {
                                  each waiting for its group's previous unit, so work moves
                                  between SMs and no SM finishes late because it holds one warp
                                  more than another.  Used for launches of at least 4 units per
-                                 warp-group and more than 8 warps per SM (others run as plain
+                                 warp-group and more than 8 warps per SM, or 128 where planet
+                                 counts differ and block_size is 0 (others run as plain
                                  launches); queue launches use one-warp blocks (block_size does
                                  not apply).  0: one warp per warp-group for the whole launch.
                                  Results are bitwise the same either way.  A wait that exceeds

@@ -105,6 +105,7 @@ WhgLaunch launch_cfg(const whg_ctx* c)
     if (l.grid < 1) l.grid = 1;
     l.stream = c->stream;
     l.sms = 0;
+    l.auto_block = c->opt.block_size == 0;
     return l;
 }
 
@@ -245,7 +246,7 @@ constexpr long long kQueueSpinLimit = 1LL << 26;
 cudaError_t launch_steps(whg_ctx* c, long long n_steps, const WhgLaunch& l)
 {
     const long long qs = c->opt.queue_steps;
-    if (!c->q_next || n_steps < kQueueMinUnits * qs || whg_few_warps(c->bk))
+    if (!c->q_next || n_steps < kQueueMinUnits * qs || whg_plain_steps(c->bk, l))
         return whg_launch_step(c->st, c->bk, n_steps, c->opt.newton_terms, c->opt.gr_mode, l);
     WhgQueue q{c->q_next, c->q_done, c->q_err, qs, (int)((n_steps + qs - 1) / qs), kQueueSpinLimit};
     cudaError_t e = cudaMemsetAsync(c->q_next, 0, sizeof(unsigned long long), l.stream);
@@ -942,6 +943,7 @@ static WhgLaunch chain_cfg(const whg_ctx* c, bool on_split)
         if (l.grid < 1) l.grid = 1;
         l.stream = c->s_chain;
         l.sms = c->chain_sms;
+        l.auto_block = false;
     }
     return l;
 }

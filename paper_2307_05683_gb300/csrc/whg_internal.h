@@ -127,6 +127,7 @@ struct WhgLaunch {
     int grid, block;
     cudaStream_t stream;
     int sms;                         // SMs the launch has (0: all of the device's)
+    bool auto_block;                 // the step kernels may take larger blocks than `block`
 };
 
 // Warps of bucket b, and of all buckets, with four lanes per planet (whg_wide.cuh).
@@ -155,9 +156,8 @@ cudaError_t whg_launch_repack(const WhgState& st, const WhgState& scratch, const
 cudaError_t whg_launch_raw(const WhgState&, const WhgBuckets&, const WhgOut&, int set, const WhgLaunch&);
 cudaError_t whg_launch_step(const WhgState&, const WhgBuckets&, long long nsteps, int newton_terms,
                             int gr_mode, const WhgLaunch&);
-// Whether an ensemble's warps leave every SM at most 8 of them: such launches run
-// the step kernel built for few warps, and have no use for the work queue.
-bool whg_few_warps(const WhgBuckets&);
+// Whether step launches of this shape have no use for the work queue.
+bool whg_plain_steps(const WhgBuckets&, const WhgLaunch&);
 // Step kernel over the work queue (q.next and q.done zeroed by the caller).
 cudaError_t whg_launch_step_queue(const WhgState&, const WhgBuckets&, long long nsteps, int newton_terms,
                                   int gr_mode, const WhgQueue& q, cudaStream_t stream);

@@ -185,20 +185,48 @@ static bool wide_warps(const WhgState& st, const WhgBuckets& bk, int sms)
     return whg_wide_warps(bk) <= (least >= 6 ? 12 : 8) * sms;
 }
 
-bool whg_few_warps(const WhgBuckets& bk) { return bk.warp0[bk.nb] <= 8 * sm_count(); }
+// Blocks for an ensemble of several lane-group sizes: as many consecutive warps,
+// which are of one size but for the bucket borders, as make one block per SM, at
+// most 8.  Every size has its own unrolled step of ~35 KB of code, and with one-warp
+// blocks, dealt out over the SMs, each SM ran most of them side by side, more than
+// its instruction cache holds.  us per step, compact systems of 2 to 8 planets,
+// one-warp blocks / these: 300 2.9 / 2.6, 1500 10.4 / 3.3, 4096 11.9 / 4.8, 7000
+// 14.3 / 5.9, 12,000 16.9 / 9.0, 65,536 37.1 / 36.9; 4096 of them at steps of P/7, with
+// a few systems redone in FP64 each step, 18.0 / 5.0 (15.8 when all was FP64).
+static WhgLaunch mixed_blocks(const WhgLaunch& l, const WhgBuckets& bk, int warps, int sms)
+{
+    WhgLaunch m = l;
+    if (!l.auto_block || bk.nb < 2 || sms < 1) return m;
+    const int per = (warps + sms - 1) / sms, w = per < 1 ? 1 : (per < WHG_MAX_BLOCK / 32 ? per : WHG_MAX_BLOCK / 32);
+    m.block = 32 * w;
+    m.grid = (warps + w - 1) / w;
+    return m;
+}
+
+// The work queue balances SMs, but deals one-warp units of every lane-group size to
+// all of them.  Ensembles of several sizes do without up to 128 warps per SM: us per
+// step, queue / blocks as above: 9000 compact systems 18.3 / 8.2, 20,000 19.7 / 13.5,
+// 65,536 39.1 / 36.7, 200,000 (217 warps per SM) 103.2 / 104.3.
+bool whg_plain_steps(const WhgBuckets& bk, const WhgLaunch& l)
+{
+    return bk.warp0[bk.nb] <= (l.auto_block && bk.nb > 1 ? 128 : 8) * sm_count();
+}
 
 cudaError_t whg_launch_step(const WhgState& st, const WhgBuckets& bk, long long n, int newton_terms,
                             int gr_mode, const WhgLaunch& l)
 {
     const int sms = l.sms > 0 ? l.sms : sm_count();
-    if (wide_warps(st, bk, sms))
-        return newton_terms == 6 ? whg_launch_step_wide_nt6(st, bk, n, gr_mode, l)
-                                 : whg_launch_step_wide_nt8(st, bk, n, gr_mode, l);
-    if (bk.warp0[bk.nb] <= 8 * sms)
-        return newton_terms == 6 ? whg_launch_step_few_nt6(st, bk, n, gr_mode, l)
-                                 : whg_launch_step_few_nt8(st, bk, n, gr_mode, l);
-    return newton_terms == 6 ? whg_launch_step_nt6(st, bk, n, gr_mode, l)
-                             : whg_launch_step_nt8(st, bk, n, gr_mode, l);
+    const bool wide = wide_warps(st, bk, sms);
+    const int warps = wide ? whg_wide_warps(bk) : bk.warp0[bk.nb];
+    const WhgLaunch m = mixed_blocks(l, bk, warps, sms);
+    if (wide)
+        return newton_terms == 6 ? whg_launch_step_wide_nt6(st, bk, n, gr_mode, m)
+                                 : whg_launch_step_wide_nt8(st, bk, n, gr_mode, m);
+    if (warps <= 8 * sms)
+        return newton_terms == 6 ? whg_launch_step_few_nt6(st, bk, n, gr_mode, m)
+                                 : whg_launch_step_few_nt8(st, bk, n, gr_mode, m);
+    return newton_terms == 6 ? whg_launch_step_nt6(st, bk, n, gr_mode, m)
+                             : whg_launch_step_nt8(st, bk, n, gr_mode, m);
 }
 
 cudaError_t whg_launch_step_queue(const WhgState& st, const WhgBuckets& bk, long long n, int newton_terms,

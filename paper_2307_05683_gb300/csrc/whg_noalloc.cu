@@ -147,6 +147,7 @@ extern "C" int whg_integrate_noalloc(int n_systems, int max_planets, const whg_o
     l.grid = (int)((NL + block - 1) / block);
     l.stream = (cudaStream_t)cuda_stream;
     l.sms = 0;
+    l.auto_block = false;                            // one lane-group size
 
     // The init kernel writes every lane and per-system field read later
     // (status and step counters start at zero), so stale contents left by an

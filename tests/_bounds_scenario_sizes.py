@@ -28,8 +28,8 @@ solar, mixed = inputs.solar_ensemble(5, 2600), inputs.compact_ensemble(6, 12000)
 run("few_warps", solar, (20,), gr_mode=1)
 run("few_warps_mixed", mixed.subset(np.arange(5000)), (60,), gr_mode=2, newton_terms=6, **stop)
 run("many_warps", mixed, (30,), gr_mode=1, queue_steps=0)
-run("queue", mixed, (60, 45), gr_mode=0, queue_steps=10)
-run("queue_stop_repack_graph", mixed, (300,), gr_mode=1, queue_steps=20, repack_frozen=True, steps_per_launch=100,
+run("queue", mixed, (60, 45), gr_mode=0, queue_steps=10, block_size=32)
+run("queue_stop_repack_graph", mixed, (300,), gr_mode=1, queue_steps=20, block_size=32, repack_frozen=True, steps_per_launch=100,
     graph_launches=2, **stop)
 run("four_lanes_mixed", mixed.subset(np.arange(300)), (60,), gr_mode=2, **stop)
 

@@ -53,11 +53,24 @@ def test_queue_with_stop_rules_graphs_and_repacking(whg, extra):
     of 37 and 25 steps, two calls."""
     ens = inputs.compact_ensemble(46, 12000)
     assert _many_warps(ens)
-    kw = dict(close_encounter_hill=8.0, eject_factor=3.0, **extra)
+    kw = dict(close_encounter_hill=8.0, eject_factor=3.0, block_size=32, **extra)
     plain = _outputs(whg, ens, (500, 160), queue_steps=0, **kw)
     assert 200 < int((plain[2] != 0).sum()) < 11800
     for unit in (37, 25):
         assert _same(plain, _outputs(whg, ens, (500, 160), queue_steps=unit, **kw)), unit
+
+
+@pytest.mark.parametrize("S", [3, 300, 1500, 2500, 5000, 7000, 12000])
+@pytest.mark.parametrize("extra", [{}, {"graph_launches": 3, "steps_per_launch": 20, "close_encounter_hill": 8.0,
+                                        "gr_mode": 2, "newton_terms": 6}])
+def test_blocks_for_several_planet_counts(whg, S, extra):
+    """Automatic blocks of 1 to 8 warps (several lane-group sizes in an ensemble,
+    block borders inside buckets and across them) against one-warp blocks, and
+    the queue, which they replace up to 128 warps per SM."""
+    ens = inputs.compact_ensemble(47, S)
+    one = _outputs(whg, ens, (90, 410), block_size=32, **extra)
+    assert _same(one, _outputs(whg, ens, (90, 410), **extra))
+    assert _same(one, _outputs(whg, ens, (90, 410), block_size=160, queue_steps=0, **extra))
 
 
 def test_queue_units_and_short_launches(whg):
