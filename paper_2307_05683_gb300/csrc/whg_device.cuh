@@ -820,9 +820,7 @@ __device__ __forceinline__ Masses<L> masses_of(const Group<L>& g, bool real, dou
 
 // The sub-step in FP64, for the systems that the float-pair form leaves out
 // (and the interaction schedule without reactions).  Out of line: few systems
-// need it, but their warp runs both forms, and where a launch has one warp per
-// sub-partition it waits for such a warp (4096 compact systems at steps of P/7, four
-// of them redone each step: 17.9 us per step against 11.8 at P/20).
+// need it.  Their warp runs both forms.
 // Warp shuffles inside: every lane calls it.
 struct SubStep {
     double m, hm, mrat, jc, kgr;
