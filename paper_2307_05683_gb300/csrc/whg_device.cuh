@@ -988,7 +988,7 @@ __device__ __forceinline__ bool interact_pairs(const Group<L>& g, const Masses<L
             k.h = pairs::mul(c.kgp.h, sc);
             k.l = pairs::mul(c.kgp.l, sc);
             const pairs::Pair w = pairs::product(k, pairs::inverse_fourth(s));
-                        const float vg = gr_scale(vl, e, c.jm, K2);
+            const float vg = gr_scale(vl, e, c.jm, K2);
             ok = ok & accept(s, -w.h, GRM == 1 ? vg : vl);
             pairs::Pair fx = pairs::product(w, s.x), fy = pairs::product(w, s.y), fz = pairs::product(w, s.z);
             if (GRM == 2) {                              // minus the mass-weighted sum, on every planet
